@@ -28,18 +28,20 @@ struct ApplyArgs {
   const float2* in;        // forward: g [nrhs][n_in]; adjoint: u [nrhs][n_out]
   float2* out;             // forward: u; adjoint: g
   int64_t in_len, out_len;
-  float2* bufs;            // stage e writes bufs + e * buf_stride ([pos][NRB]); stage e+1 reads it
+  float2* bufs;            // stage e < S - 1 writes bufs + e * buf_stride ([pos][NRB]); stage e+1 reads it
   int64_t buf_stride;
   unsigned int* counters;  // [stage][group]: input segments written so far (zeroed per launch)
-  unsigned int* barrier;   // grid barrier between passes (zeroed per launch)
   int* status;             // 0 = ok; nonzero = a device wait ran out of time (sticky)
-  int32_t nrhs, n_pass, n_slots;
+  int32_t nrhs, rhs0;      // this launch applies RHS rhs0 .. min(nrhs, rhs0 + NRB) - 1
+  int32_t xcap;            // most entries of a block side or points of a leaf group (<= 256)
+  // set by the launch: ring slots; partial-sum entries; shift of the CTAs' groups per stage
+  int32_t n_slots, redcap, rot;
   int32_t accumulate;      // 1: out += result (the caller initialised out), 0: out = result
   // Failure-detection test hook (mbf_op_debug_stall); zero leaves the apply unchanged.
   // stall_stage1 = 1 + s: the dependency wait of group 0 of stage s (execution order)
   // waits for one more producer than exists, so that it can only end by running out of
-  // time.  wait_ns > 0: every wait on a dependency counter, the pass barrier or a chunk
-  // gives up after wait_ns instead of kTimeoutNs.
+  // time.  wait_ns > 0: a wait on a dependency counter gives up after wait_ns instead of
+  // kTimeoutNs, the waits inside a CTA after twice as long.
   uint64_t wait_ns;
   int32_t stall_stage1, stall_pad_;
   int32_t use_rows, rows_pad_;   // 1: in / out rows from `rows` (nrhs <= kRowTab)
@@ -108,10 +110,11 @@ struct LeafArgs {
   RowTable rows;
 };
 
-size_t simt_smem_bytes(int nrb, int ns);
-int simt_threads(int nrb);
-cudaError_t simt_config(int nrb, int* grid, int* ns, size_t* smem);
-cudaError_t launch_apply_simt(const ApplyArgs& a, int nrb, bool adj, int grid, size_t smem,
+// FP32 SIMT path (apply_simt.cu): one launch per pass of 1, 2, 4 or 8 RHS.
+int simt_threads();
+int simt_pass_rhs(int64_t rhs_left);   // RHS of the next pass (the last one may be padded)
+cudaError_t simt_config(int nrb, int xcap, SimtConfig cfg[2]);
+cudaError_t launch_apply_simt(const ApplyArgs& a, int nrb, bool adj, int sms, const SimtConfig cfg[2],
                               cudaStream_t stream);
 // Bytes of dependency counters for a plan (S stages x groups, rounded up to 256).
 size_t counter_bytes(const Plan& plan);

@@ -1,5 +1,5 @@
 // Allocation-free forward apply: the persistent FP32 kernel of apply_simt.cu run
-// with its coefficient workspace and grid-barrier counter placed in one fixed,
+// with its coefficient workspace and dependency counters placed in one fixed,
 // library-global device array instead of the operator's own workspace.
 //
 // Why: some callers may not allocate device memory when they apply an operator --
@@ -14,8 +14,8 @@
 // dependency counter per group of every stage, and one coefficient vector of
 // (c^L * max rank) entries per stage for each of up to 4 RHS per pass; larger needs
 // are rejected with MBF_ERR_INVALID.  Every call on a device
-// shares the one array and leaves its contents behind; the barrier counter is
-// cleared at the start of each call.  Calls that overlap on the GPU (on different
+// shares the one array and leaves its contents behind; the counters are cleared at
+// the start of each pass.  Calls that overlap on the GPU (on different
 // streams, or with an mbf_apply_static on another operator) race on the array.
 #include <cuda_runtime.h>
 
@@ -93,17 +93,18 @@ void apply_static_impl(mbf_op_s* op, const void* g, void* u, int64_t nrhs, void*
   a.out = static_cast<float2*>(u);
   a.in_len = op->n_in;
   a.out_len = op->n_out;
-  a.barrier = reinterpret_cast<unsigned*>(base);            // barrier + counters, cleared by the launch
-  a.counters = a.barrier + kBarrierBytes / sizeof(unsigned);
+  a.counters = reinterpret_cast<unsigned*>(base + kBarrierBytes);   // cleared by each launch
   a.bufs = reinterpret_cast<float2*>(base + sync_bytes);     // one vector per stage
   a.buf_stride = op->positions * nrb;
   a.status = op->ws.status;
   a.nrhs = int32_t(nrhs);
-  a.n_pass = int32_t((nrhs + nrb - 1) / nrb);
-  a.n_slots = op->ns[nrb];
+  a.xcap = op->xcap;
   a.plan = op->plan;
-  e = mbf::launch_apply_simt(a, nrb, false, op->grid, op->smem[nrb], static_cast<cudaStream_t>(stream));
-  if (e != cudaSuccess) mbf::fail(MBF_ERR_CUDA, std::string("apply launch: ") + cudaGetErrorString(e));
+  for (int64_t r0 = 0; r0 < nrhs; r0 += nrb) {
+    a.rhs0 = int32_t(r0);
+    e = mbf::launch_apply_simt(a, nrb, false, op->sms, op->simt[nrb], static_cast<cudaStream_t>(stream));
+    if (e != cudaSuccess) mbf::fail(MBF_ERR_CUDA, std::string("apply launch: ") + cudaGetErrorString(e));
+  }
 }
 
 }  // namespace

@@ -5,8 +5,8 @@
 //   H-stages l = L-1 .. h  apply (H^l)^*   (the first also applies (V^L)^* to the leaves)
 //   G-stages l = h .. L-1  apply G^l       (the first folds in M^h; the last applies U^L)
 // Each stage is a batch of c^(L-1) independent *group* products: one dense
-// (c R_out) x (c R_in) complex block times a gathered input of c segments.  The
-// groups of one stage are separated from the next stage by a grid-wide barrier.
+// (c R_out) x (c R_in) complex block times a gathered input of c segments.  A group
+// starts when its c input segments have been counted in (no barrier between stages).
 //
 // Factor data lives in one arena.  Each group owns a contiguous run of *items*
 // (its main block, plus c leaf blocks in the first/last stage), each item a set of
@@ -15,6 +15,7 @@
 // A main block's lines are its inputs (segment t, entry k); a compact stage stores
 // only the lines below each input segment's rank (Stage::compact).
 #pragma once
+#include <cstddef>
 #include <cstdint>
 
 #if defined(__CUDACC__)
@@ -98,6 +99,12 @@ struct TCPlan {
 
 constexpr int kTcMaxRows = 256;   // M_t limit (the MMA's N)
 constexpr int kTcMaxK = 256;      // K_t limit
+
+// A launch shape of the SIMT kernel: ring slots (0: does not fit) and shared memory of a CTA.
+struct SimtConfig {
+  int slots = 0;
+  size_t smem = 0;
+};
 
 // Byte of an item's base holding r_t in a compact stage.
 MBF_HD int seg_lines(int32_t base, int t) { return int((uint32_t(base) >> (8 * t)) & 0xffu); }

@@ -651,7 +651,13 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
     op->d_x_nat = dev_upload(nat_table(f.x_perm, f.x_off, op->leaf_pts_x, &op->x_nat_stride), "X leaf index table");
     op->d_w_nat = dev_upload(nat_table(f.w_perm, f.w_off, op->leaf_pts_w, &op->w_nat_stride), "Omega leaf index table");
     ws_init(op, op->ws);
-    for (int nrb : {1, 2, 4}) cuda_check(simt_config(nrb, &op->grid, &op->ns[nrb], &op->smem[nrb]), "simt_config");
+    for (const Stage& st : op->plan.st)
+      op->xcap = std::max({op->xcap, op->c * st.R_in, op->c * st.R_out});
+    for (const int64_t* off : {f.x_off, f.w_off})
+      for (int64_t gq = 0; gq < nL / op->c; ++gq)
+        op->xcap = std::max<int>(op->xcap, int(std::min<int64_t>(off[(gq + 1) * op->c] - off[gq * op->c], kMaxGroupPoints)));
+    for (int nrb : {1, 2, 4, 8})
+      cuda_check(simt_config(nrb, op->xcap, op->simt[nrb]), "simt_config");
     cuda_check(cudaDeviceGetAttribute(&op->sms, cudaDevAttrMultiProcessorCount, op->device), "attr");
     // tensor-core tiles (the multi-RHS path); an operator whose tiles do not fit keeps
     // the SIMT path only and says why
@@ -1008,7 +1014,6 @@ void apply_impl(mbf_op_s* op, const void* in, void* out, int64_t nrhs, int32_t p
     return;
   }
   if (!op->simt_unavailable.empty()) fail(MBF_ERR_INVALID, "FP32 SIMT path unavailable: " + op->simt_unavailable);
-  const int nrb = nrhs >= 4 ? 4 : (nrhs >= 2 ? 2 : 1);
   ApplyArgs a{};
   a.arena = op->d_arena;
   a.items = op->d_items;
@@ -1021,13 +1026,10 @@ void apply_impl(mbf_op_s* op, const void* in, void* out, int64_t nrhs, int32_t p
   a.in_len = adj ? op->n_out : op->n_in;
   a.out_len = adj ? op->n_in : op->n_out;
   a.bufs = w.bufs;
-  a.buf_stride = op->positions * nrb;
-  a.barrier = w.barrier;
-  a.counters = w.barrier + 64;
+  a.counters = w.counters;
   a.status = w.status;
   a.nrhs = int32_t(nrhs);
-  a.n_pass = int32_t((nrhs + nrb - 1) / nrb);
-  a.n_slots = op->ns[nrb];
+  a.xcap = op->xcap;
   a.plan = op->plan;
   a.accumulate = accumulate ? 1 : 0;
   a.wait_ns = op->dbg_wait_ns;
@@ -1038,10 +1040,16 @@ void apply_impl(mbf_op_s* op, const void* in, void* out, int64_t nrhs, int32_t p
   }
   if (adj && op->n_w < op->n_in && !accumulate)
     cuda_check(cudaMemsetAsync(out, 0, size_t(nrhs) * size_t(op->n_in) * sizeof(float2), st), "cudaMemsetAsync");
-  cudaEvent_t e0 = prof_begin(op, st);
-  const int g = grid > 0 ? std::min(grid, op->grid) : op->grid;
-  cuda_check(launch_apply_simt(a, nrb, adj, g, op->smem[nrb], st), "apply launch");
-  prof_end(op, PK_SIMT, e0, st);
+  const int sms = grid > 0 ? std::min(grid, op->sms) : op->sms;
+  for (int64_t r0 = 0; r0 < nrhs;) {
+    const int nrb = simt_pass_rhs(nrhs - r0);
+    a.rhs0 = int32_t(r0);
+    a.buf_stride = op->positions * nrb;
+    cudaEvent_t e0 = prof_begin(op, st);
+    cuda_check(launch_apply_simt(a, nrb, adj, sms, op->simt[nrb], st), "apply launch");
+    prof_end(op, PK_SIMT, e0, st);
+    r0 += nrb;
+  }
 }
 
 }  // namespace
@@ -1075,10 +1083,10 @@ int64_t tc_vec_bytes(const mbf_op_s* op) {
 // (or through tc_prepare / the server before a capture), so later applies allocate
 // nothing.
 void ws_init(const mbf_op_s* op, Workspace& w) {
-  const size_t vbytes = size_t(op->plan.n_stages) * size_t(op->positions) * 4 * sizeof(float2);
+  const size_t vbytes = size_t(op->plan.n_stages - 1) * size_t(op->positions) * 8 * sizeof(float2);
   if (dev_alloc(&w.bufs, vbytes) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc workspace");
-  if (dev_alloc(&w.barrier, 256 + counter_bytes(op->plan)) != cudaSuccess || dev_alloc(&w.status, 256) != cudaSuccess)
-    fail(MBF_ERR_OOM, "cudaMalloc barrier");
+  if (dev_alloc(&w.counters, counter_bytes(op->plan)) != cudaSuccess || dev_alloc(&w.status, 256) != cudaSuccess)
+    fail(MBF_ERR_OOM, "cudaMalloc counters");
   cuda_check(cudaMemset(w.status, 0, 256), "cudaMemset status");
 }
 
@@ -1096,7 +1104,7 @@ void ws_prepare_tc(const mbf_op_s* op, Workspace& w) {
 
 void ws_free(Workspace& w) {
   cudaFree(w.bufs);
-  cudaFree(w.barrier);
+  cudaFree(w.counters);
   cudaFree(w.status);
   cudaFree(w.tc_bufs);
   cudaFree(w.tc_counters);
@@ -1325,9 +1333,9 @@ mbf_status mbf_op_info(mbf_op_t op, mbf_op_info_t* info) {
     info->bytes_algorithmic = 8 * op->nnz;
     info->bytes_packed = op->bytes_packed;
     for (int s = 0; s < op->plan.n_stages && s < 32; ++s) info->bytes_stage[s] = op->plan.st[s].bytes;
-    info->grid = op->grid;
-    info->threads = simt_threads(1);
-    info->smem = int(op->smem[1]);
+    info->grid = op->sms;
+    info->threads = simt_threads();
+    info->smem = int(op->simt[1][0].smem);
     for (size_t e = 0; e < op->nnz_stage.size() && e < 32; ++e) info->nnz_stage[e] = op->nnz_stage[e];
     info->nnz_leaf_u = op->nnz_leaf_x;
     info->tensor_ok = op->tc_unavailable.empty() ? 1 : 0;

@@ -17,14 +17,14 @@ struct mbf_factors_s {
 namespace mbf {
 struct RowTable;   // apply.hpp
 
-// Scratch of one apply in flight: the SIMT kernel's coefficient vectors, grid-barrier
-// word and dependency counters, the status word its waits report to, and the tensor
+// Scratch of one apply in flight: the SIMT kernel's coefficient vectors and
+// dependency counters, the status word its waits report to, and the tensor
 // path's vectors, counters and tree-ordered input panel (allocated on first tensor
 // use).  An operator owns one, and lends further ones from a pool it keeps to the
 // server, so that batches of one operator can run at the same time.
 struct Workspace {
-  float2* bufs = nullptr;          // one coefficient vector per stage, 4 RHS wide
-  unsigned* barrier = nullptr;     // barrier word, then (256 bytes on) the dependency counters
+  float2* bufs = nullptr;          // one coefficient vector per stage but the last, 8 RHS wide
+  unsigned* counters = nullptr;    // the dependency counters
   int* status = nullptr;
   uint8_t* tc_bufs = nullptr;      // S_main + 1 vectors of c^L blocks x R8 x 64 entries (8 bytes each)
   unsigned* tc_counters = nullptr;
@@ -51,8 +51,10 @@ struct mbf_op_s {
   int32_t x_nat_stride = 0, w_nat_stride = 0;
   int32_t split_x = 0, split_w = 0;         // U^L-side leaf kernels: one CTA per leaf (ragged tree)
   mbf::Workspace ws;                // the scratch of the operator's own applies
-  int grid = 0, ns[5] = {0, 0, 0, 0, 0};
-  size_t smem[5] = {0, 0, 0, 0, 0};
+  // SIMT kernel: its launch shapes by RHS per pass (1, 2, 4, 8); xcap: most entries of a
+  // block side or points of a leaf group
+  mbf::SimtConfig simt[9][2];
+  int xcap = 1;
   // tensor-core path: arena of split-bf16 tiles of the main stages, its plan, and the
   // panel workspace (allocated on first use)
   mbf::TCPlan tcplan{};
