@@ -25,10 +25,17 @@
 //   warps 4-7, 8-11   epilogue sets, one per accumulator set: read the accumulators
 //              (tcgen05.ld, 32 columns of each half a round), pair the halves by warp
 //              shuffles, split and store the group's output blocks, and hand them to
-//   warp 12    the signal warp, which fences and counts them in for the consumers;
+//   warps 12, 14  the sets' signal warps, which fence and count them in for the consumers;
 //   warps 3, 13  drop each group's consumed input blocks from L2 once its MMAs are done.
 // The (V^L)^* and U^L leaf products run before and after it (leaf kernels below).
 // Every wait is bounded; on a timeout the status word is set and all roles drain.
+// What bounds it: with 64 RHS of the polar FIO n = 256 a group takes a CTA 3500 cycles (from
+// 4800): its 18 MMAs need 1730, its 74 KB of tile 3400 at the HBM copy rate, and the vectors'
+// 98 KB go through L2 besides.  The roles' own instructions mattered: ring positions and
+// output blocks are kept incrementally (a runtime division or two per chunk and per 8
+// rows was most of the MMA warp's 550 cycles per chunk), and the fence behind a group's
+// stores, 2300 cycles, overlaps the other set's and covers all groups stored by then (it
+// paced the kernel at one group per fence).  122 -> 100 us; n = 128, r = 16, 20 RHS: 87 -> 61.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
@@ -94,6 +101,15 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // Drop a 128-byte line from L2 without writing it back (its contents become undefined).
 __device__ __forceinline__ void l2_discard(const void* p) {
   asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
+}
+// Counters in shared memory between roles of a CTA.
+__device__ __forceinline__ void st_release_cta(unsigned* p, unsigned v) {
+  asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(sa(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned ld_acquire_cta(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(sa(p)) : "memory");
+  return v;
 }
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
@@ -201,13 +217,30 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
-// Block index (tree-node pair of the level) of segment t of group g under a pattern.
-__device__ __forceinline__ int64_t pat_blk(int pat, int g, int t, const TCStage& s, int c) {
-  const int a = g / s.B, b = g - (g / s.B) * s.B;
-  if (pat == PAT_SPLIT) return int64_t(c * a + t) * s.B + b;
-  if (pat == PAT_CONTIG) return int64_t(c) * g + t;
-  return int64_t(c * b + t) * s.ch + a;  // PAT_CORNER
+// Blocks (tree-node pairs of the level) of a group's segments under a pattern: segment t
+// is block base + t step.
+struct SegBlocks {
+  int base, step;
+};
+__device__ __forceinline__ SegBlocks seg_blocks(int pat, int g, const TCStage& s, int c) {
+  if (pat == PAT_CONTIG) return {c * g, 1};
+  const int a = g / s.B, b = g - a * s.B;
+  if (pat == PAT_SPLIT) return {c * a * s.B + b, s.B};
+  return {c * b * s.ch + a, s.ch};  // PAT_CORNER
 }
+// Position in a ring of n entries, kept by each role: entry and phase parity of its
+// current use (a division per step costs more than the rest of a hand-over).
+struct RingPos {
+  int i = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next(int n, int by = 1) {
+    i += by;
+    if (i >= n) {
+      i -= n;
+      ph ^= 1u;
+    }
+  }
+};
 __device__ __forceinline__ int pat_group(int pat, int64_t P, const TCStage& s, int c) {
   if (pat == PAT_CONTIG) return int(P / c);
   if (pat == PAT_SPLIT) {
@@ -233,7 +266,7 @@ __device__ __forceinline__ bool wait_bar(uint64_t* b, uint32_t ph, volatile int*
 
 }  // namespace tc
 
-constexpr int kTcThreads = 448;   // 14 warps (roles above)
+constexpr int kTcThreads = 480;   // 15 warps (roles above)
 constexpr int kAProducers = 2;    // lanes of warp 0 issuing the tile copies
 constexpr int kMaxXBufs = 3;      // panel buffers at most (the autotuner picks 2 or 3)
 constexpr int kTcChunk = 16;   // accumulator columns per epilogue step
@@ -255,10 +288,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
   uint64_t* xempty = xfull + kMaxXBufs;
   uint64_t* dfull = xempty + kMaxXBufs;
   uint64_t* dempty = dfull + 2;
-  uint64_t* stored = dempty + 2;     // [set]: the set's output blocks of a group are written
-  uint64_t* signaled = stored + 2;   // [set]: the signal warp has counted them in
-  uint64_t* done = signaled + 2;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
+  uint64_t* done = dempty + 2;
+  unsigned* nstored = reinterpret_cast<unsigned*>(done + 1);   // [set][warp]: groups whose outputs the warp has written
+  uint32_t* tslot = nstored + 8;
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -275,10 +307,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
       mbar_init(&dfull[s], 1);
       mbar_init(&dempty[s], 128);
     }
-    for (int s2 = 0; s2 < 2; ++s2) {
-      mbar_init(&stored[s2], 128);
-      mbar_init(&signaled[s2], 1);
-    }
+    for (int q = 0; q < 8; ++q) nstored[q] = 0;
     mbar_init(done, 1);
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -302,18 +331,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     // share the chunks: lane p takes chunks ca = p mod kAProducers, i.e. the ring slots
     // of that residue (nsa is a multiple of kAProducers).
     const uint64_t pol = policy_evict_first();
-    uint32_t ca = 0;
+    RingPos pos;
+    pos.i = lane;
+    uint32_t ca = 0, mine = 0;   // chunks before this group; chunks this lane issued
     bool ok = true;
     for (int e = 0; e < S && ok; ++e) {
       const TCStage& st = plan.st[e];
       const int nk = st.K_pad / 16;
       const uint32_t chunk = 4u * uint32_t(st.plane_bytes);
-      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x) {
+      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ca += uint32_t(nk)) {
         const uint8_t* src = a.arena + st.base + int64_t(g) * st.tile_bytes;
-        for (int kk = 0; kk < nk; ++kk, ++ca) {
-          if (int(ca % uint32_t(kAProducers)) != lane) continue;
-          const uint32_t slot = ca % uint32_t(nsa), ph = (ca / uint32_t(nsa)) & 1u;
-          if (!wait_bar(&aempty[slot], ph ^ 1u, abort)) {
+        for (int kk = int((uint32_t(lane) - ca) % uint32_t(kAProducers)); kk < nk; kk += kAProducers) {
+          if (!wait_bar(&aempty[pos.i], pos.ph ^ 1u, abort)) {
             if (!*abort) {
               atomicCAS(a.status, 0, ST_EMPTY_TIMEOUT);
               *abort = 1;
@@ -321,15 +350,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
             ok = false;
             break;
           }
-          mbar_expect_tx(&afull[slot], chunk);
-          bulk_g2s_hint(aring + size_t(slot) * a_slot, src + int64_t(kk) * chunk, chunk, &afull[slot], pol);
+          mbar_expect_tx(&afull[pos.i], chunk);
+          bulk_g2s_hint(aring + size_t(pos.i) * a_slot, src + int64_t(kk) * chunk, chunk, &afull[pos.i], pol);
+          pos.next(nsa, kAProducers);
+          ++mine;
         }
       }
     }
-    // wait (bounded) for every copy of this lane still in flight
-    for (uint32_t q = (ca > uint32_t(nsa) ? ca - uint32_t(nsa) : 0u); q < ca; ++q) {
-      if (int(q % uint32_t(kAProducers)) != lane) continue;
-      const uint32_t slot = q % uint32_t(nsa), ph = (q / uint32_t(nsa)) & 1u;
+    // wait (bounded) for every copy of this lane still in flight: its chunks are lane,
+    // lane + kAProducers, ..., the last nsa / kAProducers of them
+    const uint32_t depth = uint32_t(nsa / kAProducers);
+    for (uint32_t i = mine > depth ? mine - depth : 0u; i < mine; ++i) {
+      const uint32_t q = uint32_t(lane) + i * kAProducers, slot = q % uint32_t(nsa), ph = (q / uint32_t(nsa)) & 1u;
       const uint64_t t1 = gtimer();
       while (!mbar_try(&afull[slot], ph) && gtimer() - t1 < kTimeoutNs) {
       }
@@ -344,6 +376,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     // consumed blocks are dropped from L2 later, by the discard warps, once the group's
     // MMAs are done.
     int j = 0;
+    RingPos pos;
     bool ok = true;
     for (int e = 0; e < S && ok; ++e) {
       const TCStage& st = plan.st[e];
@@ -353,12 +386,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
       const uint32_t xhalf = uint32_t(st.K_pad) * 256u;     // hi or lo half of the panel buffer
       const int64_t blk = split_block_bytes(st.R8_in);
       constexpr int kParts = TF32 ? 1 : 2;
-      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++j) {
-        const int xs = j % nxb;
-        const uint32_t xu = uint32_t(j / nxb);
+      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++j, pos.next(nxb)) {
+        const int xs = pos.i;
+        const SegBlocks in = seg_blocks(st.in_pat, g, st, c);
         bool fail = false;
         if (lane == 0) {
-          fail = !wait_bar(&xempty[xs], (xu & 1u) ^ 1u, abort);
+          fail = !wait_bar(&xempty[xs], pos.ph ^ 1u, abort);
           // all c input blocks written by the previous stage
           if (!fail && e > 0) {
             const unsigned* cp = cnt_in + g;
@@ -385,7 +418,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
         }
         if (lane < kParts * c) {
           const int t = lane / kParts, hl = lane - t * kParts;
-          const uint8_t* sb = src + int64_t(pat_blk(st.in_pat, g, t, st, c)) * blk;
+          const uint8_t* sb = src + int64_t(in.base + t * in.step) * blk;
           uint8_t* xb = xbuf + size_t(xs) * x_buf;
           bulk_g2s(xb + uint32_t(hl) * xhalf + uint32_t(t) * half, sb + int64_t(hl) * half, half, &xfull[xs]);
         }
@@ -405,21 +438,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     // are neither in shared memory nor read again: their lines are dropped from L2
     // without a write-back.  Each discard takes a while, so two warps share them.
     const int dt = (warp == 3 ? 0 : 32) + lane;
-    int j = 0;
+    RingPos pos;
     bool ok = true;
     for (int e = 0; e < S && ok; ++e) {
       const TCStage& st = plan.st[e];
       const uint8_t* src = e == 0 ? a.x_in : a.bufs + int64_t(e - 1) * a.buf_stride;
       const int64_t blk = split_block_bytes(st.R8_in);
-      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++j) {
-        const int xs = j % nxb;
-        const uint32_t xu = uint32_t(j / nxb);
-        if (!__all_sync(0xffffffffu, wait_bar(&xempty[xs], xu & 1u, abort))) {
+      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, pos.next(nxb)) {
+        const SegBlocks in = seg_blocks(st.in_pat, g, st, c);
+        if (!__all_sync(0xffffffffu, wait_bar(&xempty[pos.i], pos.ph, abort))) {
           ok = false;
           break;
         }
         for (int t = 0; t < c; ++t) {
-          const uint8_t* sb = src + int64_t(pat_blk(st.in_pat, g, t, st, c)) * blk;
+          const uint8_t* sb = src + int64_t(in.base + t * in.step) * blk;
           for (int64_t q = dt; q < (blk >> 7); q += 64) l2_discard(sb + (q << 7));
         }
       }
@@ -428,8 +460,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     // ---------------------------------------------------------------- MMA issuer
     // The whole warp runs the loop, so that descriptors and addresses are warp-uniform;
     // one elected lane issues the MMAs and the commits.
-    uint32_t ca = 0;
-    int j = 0;
+    RingPos ap, xp, dp;   // tile ring, panel buffers, accumulator sets
     bool ok = true;
     const uint32_t abase = sa(aring), xbase0 = sa(xbuf);
     for (int e = 0; e < S && ok; ++e) {
@@ -446,10 +477,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
       const uint32_t ab = TF32 ? 2u : 1u;   // operand format: BF16 = 1, TF32 = 2
       const uint32_t idesc = (1u << 4) | (ab << 7) | (ab << 10) | ((nmma >> 3) << 17) | (uint32_t(128 >> 4) << 24);
       const uint32_t pbt = uint32_t(st.M_t) * 64u;   // TF32: one K16 chunk of one plane
-      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++j) {
-        const int xs = j % nxb, ds = j % nsets;
-        const uint32_t xu = uint32_t(j / nxb), du = uint32_t(j / nsets);
-        const bool got = wait_bar(&xfull[xs], xu & 1u, abort) && wait_bar(&dempty[ds], (du & 1u) ^ 1u, abort);
+      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, xp.next(nxb), dp.next(nsets)) {
+        const int xs = xp.i, ds = dp.i;
+        const bool got = wait_bar(&xfull[xs], xp.ph, abort) && wait_bar(&dempty[ds], dp.ph ^ 1u, abort);
         if (!__all_sync(0xffffffffu, got)) {
           if (lane == 0 && !*abort) {
             atomicCAS(a.status, 0, ST_FULL_TIMEOUT);
@@ -461,16 +491,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d1 = taddr + uint32_t(ds) * set_cols, d2 = d1 + uint32_t(st.M_t);
         const uint32_t xb = xbase0 + uint32_t(xs) * x_buf;
-        for (int kk = 0; kk < nk; ++kk, ++ca) {
-          const uint32_t slot = ca % uint32_t(nsa), ph = (ca / uint32_t(nsa)) & 1u;
-          if (!__all_sync(0xffffffffu, wait_bar(&afull[slot], ph, abort))) {
-            if (lane == 0 && !*abort) {
-              atomicCAS(a.status, 0, ST_FULL_TIMEOUT);
-              *abort = 1;
-            }
-            ok = false;
-            break;
-          }
+        for (int kk = 0; kk < nk; ++kk, ap.next(nsa)) {
+          const uint32_t slot = uint32_t(ap.i);
+          // (a wait that gives up is dealt with at the end of the group: until then the MMAs
+          // read whatever the slot holds, and the result is discarded)
+          ok = wait_bar(&afull[slot], ap.ph, abort) && ok;
           // (the chunk was written by the bulk copy the mbarrier tracks: no tcgen05 fence)
           const uint32_t as = abase + slot * a_slot;
           if constexpr (TF32) {
@@ -518,7 +543,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
           }
           __syncwarp();
         }
-        if (!ok) break;
+        if (!__all_sync(0xffffffffu, ok)) {
+          if (lane == 0 && !*abort) {
+            atomicCAS(a.status, 0, ST_FULL_TIMEOUT);
+            *abort = 1;
+          }
+          ok = false;
+          break;
+        }
         if (elect_one()) {
           mma_commit(&dfull[ds]);
           mma_commit(&xempty[xs]);
@@ -550,9 +582,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
       uint8_t* dst = a.bufs + int64_t(e) * a.buf_stride;
       const int64_t blk = split_block_bytes(st.R8_out);
       const uint32_t half = uint32_t(st.R8_out) * 256u;
-      // pair, split and store the 16 accumulator columns c0 .. c0 + 15 (output rows of
-      // the group) held in v1 (D1) and v2 (D2)
-      auto emit = [&](int g, int c0, const float* v1, const float* v2) {
+      // pair, split and store 16 accumulator columns (output rows of the group, from entry k2
+      // of block P on) held in v1 (D1) and v2 (D2)
+      int64_t P = 0;
+      int k2 = 0, step = 0;
+      auto emit = [&](const float* v1, const float* v2) {
         float y[kTcChunk];
 #pragma unroll
         for (int q = 0; q < kTcChunk; ++q) {
@@ -562,9 +596,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
         }
 #pragma unroll
         for (int r8 = 0; r8 < kTcChunk / 8; ++r8) {
-          const int m0 = c0 + 8 * r8;
-          const int t = m0 / st.R8_out, k2 = m0 - t * st.R8_out;
-          const int64_t P = pat_blk(st.out_pat, g, t, st, c);
           if (last) {
             float* o = a.y_out + (P * st.R_out + k2) * (2 * kTcNR) + ri * kTcNR + n;
 #pragma unroll
@@ -581,11 +612,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
             *reinterpret_cast<uint4*>(o) = hi;
             *reinterpret_cast<uint4*>(o + half) = lo;
           }
+          k2 += 8;                       // (blocks hold a multiple of 8 rows)
+          if (k2 == st.R8_out) {
+            k2 = 0;
+            P += step;
+          }
         }
       };
       for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++j) {
-        if (j % nsets != set) continue;
-        const uint32_t du = uint32_t(j / nsets);
+        if (nsets == 2 && (j & 1) != set) continue;
+        const uint32_t du = uint32_t(nsets == 2 ? j >> 1 : j);
+        const SegBlocks out = seg_blocks(st.out_pat, g, st, c);
+        P = out.base;
+        step = out.step;
+        k2 = 0;
         // wait for the MMAs of this group (every lane observes the phase)
         if (!__all_sync(0xffffffffu, wait_bar(&dfull[set], du & 1u, abort))) {
           if (lane == 0 && !*abort) {
@@ -609,51 +649,61 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(&dempty[set]);
           }
-          emit(g, c0, v1, v2);
-          emit(g, c0 + kTcChunk, v1 + kTcChunk, v2 + kTcChunk);
+          emit(v1, v2);
+          emit(v1 + kTcChunk, v2 + kTcChunk);
         }
-        // hand the written blocks to the signal warp (which counts them in for the next
-        // stage off this set's path); first make sure it took the set's previous group,
-        // so that the two never get a full phase apart
-        if (du > 0 && !wait_bar(&signaled[set], (du - 1) & 1u, abort)) {
-          if (!*abort) {
-            atomicCAS(a.status, 0, ST_FULL_TIMEOUT);
-            *abort = 1;
-          }
-        } else {
-          mbar_arrive(&stored[set]);   // release: the set's stores before the signal warp's fence
-        }
+        // tell the set's signal warp (which counts the blocks in for the next stage, off this
+        // set's path)
+        __syncwarp();
+        if (lane == 0) st_release_cta(&nstored[set * 4 + quarter], du + 1);
       }
     }
-  } else if (warp == 12) {
-    // ---------------------------------------------------------------- signal warp
-    // For each group in order: wait until its epilogue set has stored the output
-    // blocks, make them visible GPU-wide (fence) and count them in for the consumers.
+  } else if ((warp == 12 || warp == 14) && (warp - 12) / 2 < nsets) {
+    // ---------------------------------------------------------------- signal warps
+    // One per accumulator set: as soon as the set's four warps have stored a group's output
+    // blocks, make them visible GPU-wide and count them in for the consumers.  The fence
+    // waits for the SM's stores in flight (over a microsecond behind a full store path), so
+    // one fence covers every group stored by then, the two sets' fences overlap, and the
+    // epilogue never waits for one.
+    const int set = (warp - 12) / 2;
     int j = 0;
+    unsigned n = 0, avail = 0;   // groups of this set signalled; seen stored
     bool ok = true;
-    for (int e = 0; e < S && ok; ++e) {
+    for (int e = 0; e + 1 < S && ok; ++e) {
       const TCStage& st = plan.st[e];
-      const bool last = st.last != 0;
-      const TCStage& nst = plan.st[e + 1 < S ? e + 1 : e];
+      const TCStage& nst = plan.st[e + 1];
       unsigned* cnt_out = a.counters + int64_t(e + 1) * nst.n_groups;
       for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++j) {
-        const int set = j % nsets;
-        const uint32_t du = uint32_t(j / nsets);
-        if (!__all_sync(0xffffffffu, wait_bar(&stored[set], du & 1u, abort))) {
-          if (lane == 0 && !*abort) {
-            atomicCAS(a.status, 0, ST_FULL_TIMEOUT);
-            *abort = 1;
+        if (nsets == 2 && (j & 1) != set) continue;
+        const SegBlocks out = seg_blocks(st.out_pat, g, st, c);
+        const int consumer = lane < c ? pat_group(nst.in_pat, out.base + int64_t(lane) * out.step, nst, c) : 0;
+        if (n >= avail) {
+          uint64_t t0 = 0;
+          for (unsigned k = 1; (avail = ld_acquire_cta(&nstored[set * 4 + (lane & 3)])) <= n; ++k) {
+            __nanosleep(20);
+            if ((k & 63u) == 0) {
+              const uint64_t t = gtimer();
+              if (t0 == 0) t0 = t;
+              if (*abort) {
+                ok = false;
+                break;
+              }
+              if (t - t0 > kTimeoutNs) {
+                atomicCAS(a.status, 0, ST_FULL_TIMEOUT);
+                *abort = 1;
+                ok = false;
+                break;
+              }
+            }
           }
-          ok = false;
-          break;
-        }
-        if (!last && lane < c) {
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          avail = __reduce_min_sync(0xffffffffu, avail);   // what all four warps have stored
+          __syncwarp();
           __threadfence();
-          const int64_t P = pat_blk(st.out_pat, g, lane, st, c);
-          atomicAdd(cnt_out + pat_group(nst.in_pat, P, nst, c), 1u);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&signaled[set]);
+        if (lane < c) atomicAdd(cnt_out + consumer, 1u);
+        ++n;
       }
     }
   }
@@ -1049,7 +1099,7 @@ __global__ void __launch_bounds__(kLeafThreads) leaf_u_kernel(const __grid_const
 size_t tc_smem_bytes(int nsa, int nxb, int nsets, int mt_max, int kpad_max) {
   (void)nsets;
   return size_t(nsa) * 4 * size_t(mt_max) * 32 + size_t(nxb) * 2 * size_t(kpad_max) * 256 +
-         (2 * size_t(nsa) + 20) * 8 + 64;
+         (2 * size_t(nsa) + 2 * kMaxXBufs + 5) * 8 + 8 * 4 + 64;
 }
 
 size_t leaf_smem_bytes(int R, int c, bool u_side, int pts_cap) {
