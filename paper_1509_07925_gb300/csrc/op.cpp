@@ -623,8 +623,11 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
       op->leaf_pts_x = std::max(op->leaf_pts_x, f.x_off[q + 1] - f.x_off[q]);
       op->leaf_pts_w = std::max(op->leaf_pts_w, f.w_off[q + 1] - f.w_off[q]);
     }
-    // a tree whose largest group of c leaves holds more than twice the mean of the
-    // non-empty groups gets one CTA per leaf in the leaf kernels of its U^L side
+    // one CTA per leaf instead of per group of c leaves in the leaf kernels of the U^L side:
+    // for a tree whose largest group holds more than twice the mean of the non-empty ones,
+    // and where the groups alone would leave SMs idle (64 groups of 256 points, 32 RHS:
+    // 47 us a CTA per group)
+    const bool few = nL / op->c < 2 * 152;
     auto ragged = [&](const int64_t* off) {
       int64_t mx = 0, tot = 0, ne = 0;
       for (int64_t gq = 0; gq < nL / op->c; ++gq) {
@@ -635,8 +638,8 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
       }
       return ne > 0 && mx * ne > 2 * tot;
     };
-    op->split_x = ragged(f.x_off) ? 1 : 0;
-    op->split_w = ragged(f.w_off) ? 1 : 0;
+    op->split_x = few || ragged(f.x_off) ? 1 : 0;
+    op->split_w = few || ragged(f.w_off) ? 1 : 0;
     op->d_x_perm = dev_upload(to32(f.x_perm, f.n_out), "x_perm");
     op->d_x_off = dev_upload(to32(f.x_off, nL + 1), "x_off");
     op->d_w_perm = dev_upload(to32(f.w_perm, std::max<int64_t>(f.n_w, 1)), "w_perm");
