@@ -64,19 +64,26 @@ enum DeviceStatus : int {
 // as bf16 pairs hi = bf16(x), lo = bf16(x - hi), laid out as the MMA's K-major A
 // operand with the real and imaginary parts of RHS n interleaved on M (rows
 // m = 2 n + ri, ri = 0 real, 1 imaginary):
-//   byte (hl, k, m) = hl R8 256 + (k / 8) 2048 + (m / 8) 128 + (m % 8) 16 + (k % 8) 2.
-// A consumer copies each hi / lo half of a block into shared memory as it is.
-constexpr int kTcNR = 64;   // RHS per tensor-core panel
-MBF_HD int64_t split_block_bytes(int R8) { return int64_t(R8) * kTcNR * 8; }
+//   byte (hl, k, m) = hl R8 4 NR + (k / 8) 32 NR + (m / 8) 128 + (m % 8) 16 + (k % 8) 2
+// with NR the panel's RHS.  A consumer copies each hi / lo half of a block into shared
+// memory as it is.
+constexpr int kTcNR = 64;        // RHS of a tensor-core panel (MMAs of M = 128) ...
+// ... or half of them (M = 64): a panel of at most 32 RHS moves half the vector bytes, its
+// buffers take half the shared memory (so the tile ring is deeper) and its leaf products
+// are half as many.  n = 128, r = 16 with 20 RHS: 84 us with panels of 64, 77 with 32;
+// multiscale n = 128 with 32 RHS: 324 and 280; 3-D n = 32, r = 32 with 32 RHS: 252 (two ring
+// slots beside one panel buffer) and 173 (four).
+constexpr int kTcNRHalf = 32;
+MBF_HD int64_t split_block_bytes(int R8, int nr = kTcNR) { return int64_t(R8) * nr * 8; }
 // With TF32 operands the same block holds FP32 (TF32-rounded) values instead, byte
-//   (k, m) = (k / 4) 2048 + (m / 8) 128 + (m % 8) 16 + (k % 4) 4
-// (the MMA's K-major A operand for 32-bit types): the same R8 x 512 bytes.
+//   (k, m) = (k / 4) 32 NR + (m / 8) 128 + (m % 8) 16 + (k % 4) 4
+// (the MMA's K-major A operand for 32-bit types): the same R8 x 8 NR bytes.
 
 struct TCArgs {
   const uint8_t* arena;
   const uint8_t* x_in;     // input of main stage 0 (split blocks)
   uint8_t* bufs;           // output of main stage e < S - 1: bufs + e * buf_stride (split blocks)
-  float* y_out;            // output of the last main stage: row block * R + k, [re 64 | im 64] floats
+  float* y_out;            // output of the last main stage: row block * R + k, [re NR | im NR] floats
   int64_t buf_stride;      // bytes
   unsigned* counters;      // [stage][group], zeroed per launch
   int* status;
@@ -93,7 +100,7 @@ struct LeafArgs {
   const int32_t* perm;     // U^L: tree -> natural x index; permute: natural -> tree Omega index
   const int32_t* off;      // leaf offsets (tree order)
   const float2* vec;       // (V^L)^*: panel in tree order [point][64]; permute: g [nrhs][len_vec]
-  const float* wl;         // U^L: level-L coefficients, row block * R + k, [re 64 | im 64] floats
+  const float* wl;         // U^L: level-L coefficients, row block * R + k, [re NR | im NR] floats
   float2* outp;            // U^L: u [nrhs][len_out]; permute: panel in tree order
   uint8_t* outs;           // (V^L)^*: split blocks of the level-L vector (block c g + t)
   int64_t len_vec, len_out;
@@ -120,21 +127,22 @@ cudaError_t launch_apply_simt(const ApplyArgs& a, int nrb, bool adj, int sms, co
 size_t counter_bytes(const Plan& plan);
 
 // tensor-core path (apply_tc.cu)
-size_t tc_smem_bytes(int nsa, int nxb, int nsets, int mt_max, int kpad_max);
+size_t tc_smem_bytes(int nsa, int nxb, int nsets, int mt_max, int kpad_max, int nr = kTcNR);
 size_t tc_counter_bytes(const TCPlan& plan);
 // Dynamic shared memory of a leaf kernel; the (V^L)^* side stages pts_cap points a round.
-size_t leaf_smem_bytes(int R, int c, bool u_side, int pts_cap = 64);
+size_t leaf_smem_bytes(int R, int c, bool u_side, int pts_cap = 64, int nr = kTcNR);
 // Points per round of the (V^L)^* leaf kernel for leaves of at most max_leaf_points
 // points: rounded up to 8, within [8, 64].
 int leaf_pts_cap(int64_t max_leaf_points);
 bool leaf_fits(int R8, int c);   // leaf kernels: R8 <= 64, c <= 8
 // tf32: TF32 tiles and vectors (kind::tf32 MMAs), else split-BF16x3.
-cudaError_t launch_apply_tc(const TCArgs& a, int grid, size_t smem, cudaStream_t stream, bool tf32);
+// nr: RHS of the panel (kTcNR or kTcNRHalf).
+cudaError_t launch_apply_tc(const TCArgs& a, int grid, size_t smem, cudaStream_t stream, bool tf32, int nr);
 // TF32 tiles (two FP32 planes per K16 chunk) converted from n_chunks split-BF16 chunks of M_t rows.
 cudaError_t launch_tf32_tiles(const uint8_t* src, uint8_t* dst, int64_t n_chunks, int M_t, cudaStream_t stream);
 // U^L side: one CTA per group of c leaves; (V^L)^* side: one CTA per leaf (c n_groups CTAs).
 // xpose: the adjoint's leaf products (U^* from the U^L items, V from the (V^L)^* items).
-cudaError_t launch_leaf(const LeafArgs& a, bool u_side, int n_groups, cudaStream_t stream, bool tf32 = false,
+cudaError_t launch_leaf(const LeafArgs& a, bool u_side, int n_groups, cudaStream_t stream, int nr, bool tf32 = false,
                         bool xpose = false);
 // Adjoint (conjugate-transposed) split-BF16 tiles of one stage from its forward tiles.
 cudaError_t launch_adjoint_tiles(const uint8_t* src, uint8_t* dst, int n_groups, int M_t, int K_t, cudaStream_t stream);

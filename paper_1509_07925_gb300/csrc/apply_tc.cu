@@ -273,13 +273,16 @@ constexpr int kTcChunk = 16;   // accumulator columns per epilogue step
 
 // TF32: the vectors between stages are TF32 blocks (apply.hpp) and the tiles two FP32
 // planes (Re, Im) per K16 chunk; kind::tf32 MMAs of K = 8.  Otherwise split-BF16x3.
-template <bool TF32>
+// NR: RHS of the panel, 64 (M = 128) or 32 (M = 64).
+template <bool TF32, int NR>
 __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_constant__ TCArgs a) {
   using namespace tc;
+  constexpr uint32_t kRow = 4u * NR;     // bytes of one k of a panel half (2 NR bf16 rows)
+  constexpr uint32_t kCore = 32u * NR;   // bytes of a column of core matrices (8 bf16 or 4 TF32 of K)
   extern __shared__ __align__(1024) uint8_t smem[];
   const int nsa = a.nsa, nxb = a.nxb, nsets = a.nsets;
   const uint32_t a_slot = 4u * uint32_t(a.mt_max) * 32u;       // one K16 chunk of a tile (4 planes)
-  const uint32_t x_buf = 2u * uint32_t(a.kpad_max) * 256u;      // hi + lo halves of a panel
+  const uint32_t x_buf = 2u * uint32_t(a.kpad_max) * kRow;      // hi + lo halves of a panel
   uint8_t* aring = smem;
   uint8_t* xbuf = aring + size_t(nsa) * a_slot;
   uint64_t* afull = reinterpret_cast<uint64_t*>(xbuf + size_t(nxb) * x_buf);
@@ -382,9 +385,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
       const TCStage& st = plan.st[e];
       const uint8_t* src = e == 0 ? a.x_in : a.bufs + int64_t(e - 1) * a.buf_stride;
       const unsigned* cnt_in = a.counters + int64_t(e) * st.n_groups;
-      const uint32_t half = TF32 ? uint32_t(st.R8_in) * 512u : uint32_t(st.R8_in) * 256u;
-      const uint32_t xhalf = uint32_t(st.K_pad) * 256u;     // hi or lo half of the panel buffer
-      const int64_t blk = split_block_bytes(st.R8_in);
+      const uint32_t half = uint32_t(st.R8_in) * (TF32 ? 2u * kRow : kRow);
+      const uint32_t xhalf = uint32_t(st.K_pad) * kRow;     // hi or lo half of the panel buffer
+      const int64_t blk = split_block_bytes(st.R8_in, NR);
       constexpr int kParts = TF32 ? 1 : 2;
       for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++j, pos.next(nxb)) {
         const int xs = pos.i;
@@ -443,7 +446,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     for (int e = 0; e < S && ok; ++e) {
       const TCStage& st = plan.st[e];
       const uint8_t* src = e == 0 ? a.x_in : a.bufs + int64_t(e - 1) * a.buf_stride;
-      const int64_t blk = split_block_bytes(st.R8_in);
+      const int64_t blk = split_block_bytes(st.R8_in, NR);
       for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, pos.next(nxb)) {
         const SegBlocks in = seg_blocks(st.in_pat, g, st, c);
         if (!__all_sync(0xffffffffu, wait_bar(&xempty[pos.i], pos.ph, abort))) {
@@ -466,16 +469,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     for (int e = 0; e < S && ok; ++e) {
       const TCStage& st = plan.st[e];
       const int nk = st.K_pad / 16;
-      const uint32_t xhalf = uint32_t(st.K_pad) * 256u;
+      const uint32_t xhalf = uint32_t(st.K_pad) * kRow;
       const uint32_t pb = uint32_t(st.plane_bytes);
-      // kind::f16, FP32 accumulate, BF16 A and B, both K-major, M = 128.  While 2 M_t <= 256
+      // kind::f16, FP32 accumulate, BF16 A and B, both K-major, M = 2 NR.  While 2 M_t <= 256
       // the Re and Im planes of the tile form one B operand of N = 2 M_t rows (three MMAs
       // per K16 fill D1 | D2 at once); wider tiles take N = M_t, one MMA per plane.
       // (TF32: kind::tf32, A and B TF32, K = 8 per MMA; planes Re, Im of M_t x 16 FP32)
       const bool stack = 2 * st.M_t <= 256;
       const uint32_t nmma = uint32_t(stack ? 2 * st.M_t : st.M_t);
       const uint32_t ab = TF32 ? 2u : 1u;   // operand format: BF16 = 1, TF32 = 2
-      const uint32_t idesc = (1u << 4) | (ab << 7) | (ab << 10) | ((nmma >> 3) << 17) | (uint32_t(128 >> 4) << 24);
+      const uint32_t idesc = (1u << 4) | (ab << 7) | (ab << 10) | ((nmma >> 3) << 17) | (uint32_t(2 * NR >> 4) << 24);
       const uint32_t pbt = uint32_t(st.M_t) * 64u;   // TF32: one K16 chunk of one plane
       for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, xp.next(nxb), dp.next(nsets)) {
         const int xs = xp.i, ds = dp.i;
@@ -499,11 +502,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
           // (the chunk was written by the bulk copy the mbarrier tracks: no tcgen05 fence)
           const uint32_t as = abase + slot * a_slot;
           if constexpr (TF32) {
-            // A: K-major, 4 K (16 bytes) per core matrix: next 4 K at +2048, next 8 rows at
-            // +128; chunk kk at +8192, its second K = 8 at +4096.  B: planes 0 Re, 1 Im,
+            // A: K-major, 4 K (16 bytes) per core matrix: next 4 K at +kCore, next 8 rows at
+            // +128; chunk kk at +4 kCore, its second K = 8 at +2 kCore.  B: planes 0 Re, 1 Im,
             // next 4 K at +128, next 8 rows at +512; second K = 8 at +256.
-            const uint64_t x0 = sdesc(xb + uint32_t(kk) * 8192u, 2048u, 128u);
-            const uint64_t x1 = sdesc(xb + uint32_t(kk) * 8192u + 4096u, 2048u, 128u);
+            const uint64_t x0 = sdesc(xb + uint32_t(kk) * 4u * kCore, kCore, 128u);
+            const uint64_t x1 = sdesc(xb + uint32_t(kk) * 4u * kCore + 2u * kCore, kCore, 128u);
             const uint64_t r0 = sdesc(as, 128u, 512u), r1 = sdesc(as + 256u, 128u, 512u);
             const uint64_t i0 = sdesc(as + pbt, 128u, 512u), i1 = sdesc(as + pbt + 256u, 128u, 512u);
             const uint32_t acc0 = kk > 0 ? 1u : 0u;
@@ -519,9 +522,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
             __syncwarp();
             continue;
           }
-          // A: panel half (hi / lo), K-major, next 8 K at +2048, next 8 rows at +128
-          const uint64_t xh = sdesc(xb + uint32_t(kk) * 4096u, 2048u, 128u);
-          const uint64_t xl = sdesc(xb + xhalf + uint32_t(kk) * 4096u, 2048u, 128u);
+          // A: panel half (hi / lo), K-major, next 8 K at +kCore, next 8 rows at +128
+          const uint64_t xh = sdesc(xb + uint32_t(kk) * 2u * kCore, kCore, 128u);
+          const uint64_t xl = sdesc(xb + xhalf + uint32_t(kk) * 2u * kCore, kCore, 128u);
           // B: tile planes 0 Re hi, 1 Im hi, 2 Re lo, 3 Im lo; next 8 K at +128, next 8 rows at +256
           const uint64_t t0 = sdesc(as, 128u, 256u), t1 = sdesc(as + pb, 128u, 256u);
           const uint64_t t2 = sdesc(as + 2u * pb, 128u, 256u), t3 = sdesc(as + 3u * pb, 128u, 256u);
@@ -566,12 +569,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     }
   } else if (warp >= 4 && (warp - 4) / 4 < nsets) {
     // ---------------------------------------------------------------- epilogue sets
-    // TMEM lane tl is row tl of the panel: RHS n = tl / 2, real (ri = 0) or imaginary
-    // (ri = 1) part, so the two halves of a complex output sit in adjacent lanes of one
-    // warp and pair by a shuffle.  Each warp works on its own.
+    // Row tl of the panel: RHS n = tl / 2, real (ri = 0) or imaginary (ri = 1) part, so the
+    // two halves of a complex output sit in adjacent lanes of one warp and pair by a
+    // shuffle.  With M = 128 row tl is TMEM lane tl; with M = 64 a warp's quarter holds 16
+    // rows in its first 16 lanes.  Each warp works on its own.
     const int set = (warp - 4) >> 2;             // 0: warps 4-7, 1: warps 8-11
     const int quarter = warp & 3;                // TMEM lane quarter this warp may access
-    const int tl = quarter * 32 + lane;
+    const int tl = NR == 64 ? quarter * 32 + lane : quarter * 16 + (lane & 15);
+    const bool lane_on = NR == 64 || lane < 16;
     const int ri = tl & 1, n = tl >> 1;
     const uint32_t lane_base = uint32_t(32 * quarter) << 16;
     int j = 0;
@@ -580,8 +585,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
       const TCStage& st = plan.st[e];
       const bool last = st.last != 0;
       uint8_t* dst = a.bufs + int64_t(e) * a.buf_stride;
-      const int64_t blk = split_block_bytes(st.R8_out);
-      const uint32_t half = uint32_t(st.R8_out) * 256u;
+      const int64_t blk = split_block_bytes(st.R8_out, NR);
+      const uint32_t half = uint32_t(st.R8_out) * kRow;
       // pair, split and store 16 accumulator columns (output rows of the group, from entry k2
       // of block P on) held in v1 (D1) and v2 (D2)
       int64_t P = 0;
@@ -597,20 +602,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
 #pragma unroll
         for (int r8 = 0; r8 < kTcChunk / 8; ++r8) {
           if (last) {
-            float* o = a.y_out + (P * st.R_out + k2) * (2 * kTcNR) + ri * kTcNR + n;
+            float* o = a.y_out + (P * st.R_out + k2) * (2 * NR) + ri * NR + n;
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-              if (k2 + i < st.R_out) o[i * 2 * kTcNR] = y[8 * r8 + i];
-          } else if (TF32) {   // two runs of 4 rows: byte (k / 4) 2048 + (m / 8) 128 + (m % 8) 16
-            uint8_t* o = dst + P * blk + (k2 >> 2) * 2048 + (tl >> 3) * 128 + (tl & 7) * 16;
-            *reinterpret_cast<uint4*>(o) = tf32x4(y + 8 * r8);
-            *reinterpret_cast<uint4*>(o + 2048) = tf32x4(y + 8 * r8 + 4);
+              if (lane_on && k2 + i < st.R_out) o[i * 2 * NR] = y[8 * r8 + i];
+          } else if (TF32) {   // two runs of 4 rows: byte (k / 4) kCore + (m / 8) 128 + (m % 8) 16
+            uint8_t* o = dst + P * blk + (k2 >> 2) * kCore + (tl >> 3) * 128 + (tl & 7) * 16;
+            if (lane_on) {
+              *reinterpret_cast<uint4*>(o) = tf32x4(y + 8 * r8);
+              *reinterpret_cast<uint4*>(o + kCore) = tf32x4(y + 8 * r8 + 4);
+            }
           } else {
             uint4 hi, lo;
             split8(y + 8 * r8, hi, lo);
-            uint8_t* o = dst + P * blk + (k2 >> 3) * 2048 + (tl >> 3) * 128 + (tl & 7) * 16;
-            *reinterpret_cast<uint4*>(o) = hi;
-            *reinterpret_cast<uint4*>(o + half) = lo;
+            uint8_t* o = dst + P * blk + (k2 >> 3) * kCore + (tl >> 3) * 128 + (tl & 7) * 16;
+            if (lane_on) {
+              *reinterpret_cast<uint4*>(o) = hi;
+              *reinterpret_cast<uint4*>(o + half) = lo;
+            }
           }
           k2 += 8;                       // (blocks hold a multiple of 8 rows)
           if (k2 == st.R8_out) {
@@ -798,7 +807,7 @@ __global__ void __launch_bounds__(kLeafThreads) permute_in_kernel(const __grid_c
 
 // Rows k0 .. k0 + 7 of column n of split block `leaf` from 8 accumulators: byte
 // (hl, k, ri, n) as in apply.hpp, so 8 consecutive k are one 16-byte run per plane.
-template <bool TF32>
+template <bool TF32, int NR>
 __device__ __forceinline__ void store_split8(uint8_t* outs, int64_t leaf, int R8, int n, int k0, float2 (&acc)[8]) {
   float re[8], im[8];
 #pragma unroll
@@ -810,18 +819,19 @@ __device__ __forceinline__ void store_split8(uint8_t* outs, int64_t leaf, int R8
   // rows m = 2 n (real part) and 2 n + 1 (imaginary part) of the block: adjacent 16-byte
   // rows of one core matrix
   const int m = 2 * n;
-  if constexpr (TF32) {   // TF32 block: byte (k / 4) 2048 + (m / 8) 128 + (m % 8) 16 + (k % 4) 4
-    uint8_t* o = outs + leaf * split_block_bytes(R8) + (k0 >> 2) * 2048 + (m >> 3) * 128 + (m & 7) * 16;
+  constexpr int kCore = 32 * NR;
+  if constexpr (TF32) {   // TF32 block: byte (k / 4) kCore + (m / 8) 128 + (m % 8) 16 + (k % 4) 4
+    uint8_t* o = outs + leaf * split_block_bytes(R8, NR) + (k0 >> 2) * kCore + (m >> 3) * 128 + (m & 7) * 16;
     *reinterpret_cast<uint4*>(o) = tc::tf32x4(re);
-    *reinterpret_cast<uint4*>(o + 2048) = tc::tf32x4(re + 4);
+    *reinterpret_cast<uint4*>(o + kCore) = tc::tf32x4(re + 4);
     *reinterpret_cast<uint4*>(o + 16) = tc::tf32x4(im);
-    *reinterpret_cast<uint4*>(o + 2048 + 16) = tc::tf32x4(im + 4);
+    *reinterpret_cast<uint4*>(o + kCore + 16) = tc::tf32x4(im + 4);
   } else {
     uint4 rh, rl, ih, il;
     tc::split8(re, rh, rl);
     tc::split8(im, ih, il);
-    uint8_t* o = outs + leaf * split_block_bytes(R8) + (k0 >> 3) * 2048 + (m >> 3) * 128 + (m & 7) * 16;
-    const int64_t half = int64_t(R8) * 256;
+    uint8_t* o = outs + leaf * split_block_bytes(R8, NR) + (k0 >> 3) * kCore + (m >> 3) * 128 + (m & 7) * 16;
+    const int64_t half = int64_t(R8) * 4 * NR;
     *reinterpret_cast<uint4*>(o) = rh;               // Re hi
     *reinterpret_cast<uint4*>(o + 16) = ih;          // Im hi
     *reinterpret_cast<uint4*>(o + half) = rl;        // Re lo
@@ -829,8 +839,8 @@ __device__ __forceinline__ void store_split8(uint8_t* outs, int64_t leaf, int R8
   }
 }
 
-// (V^L)^* for a panel of 64 RHS, one CTA of 64 R8 / 8 threads per leaf j (of group
-// g = j / c):
+// (V^L)^* for a panel of NR = 64 or 32 RHS, one CTA of NR R8 / 8 threads per leaf j (of
+// group g = j / c):
 //   y_j[k][n] = sum over the points b of leaf j of conj(V^L_j[b][k]) gt[b][n],
 // gt = the panel in tree order (permute_in_kernel), stored as split block j (rows k >= R
 // are zero).  The group's item holds conj(V) with line = point (tree order from the
@@ -860,13 +870,12 @@ __device__ __forceinline__ void leaf_v_point(float2 (&acc)[8], const float2* vro
 
 // XPOSE (the adjoint's U^* leaf products): the group's item is a U^L item (line = k,
 // entry = point of the group, U itself), read transposed and conjugated.
-template <bool TF32, bool XPOSE>
-__global__ void __launch_bounds__(kTcNR * kLeafMaxR8 / 8) leaf_v_kernel(const __grid_constant__ LeafArgs a) {
+template <bool TF32, bool XPOSE, int NR>
+__global__ void __launch_bounds__(NR * kLeafMaxR8 / 8) leaf_v_kernel(const __grid_constant__ LeafArgs a) {
   using tc::sa;
   using tc::cp_async16;
   using tc::cp_async_wait_all;
   using tc::l2_discard;
-  constexpr int NR = kTcNR;
   extern __shared__ __align__(16) float2 lsm[];
   __shared__ int nat[kLeafPts];            // gather: natural indices of the round's points
   const int j = blockIdx.x, c = a.c, g = j / c, R = a.R, R8 = a.R8, cap = a.pts_cap;
@@ -895,7 +904,7 @@ __global__ void __launch_bounds__(kTcNR * kLeafMaxR8 / 8) leaf_v_kernel(const __
       if (a.gather) {
         // the round's points straight from g in natural order: thread q reads RHS
         // q / nb of point q % nb, so that a warp's loads fall on a few nearby rows
-        for (int q = tid; q < nb; q += nth) nat[q] = b0 == 0 ? nat0 : __ldg(natj + b0 + q);
+        for (int q = tid; q < nb; q += nth) nat[q] = b0 == 0 && q == tid ? nat0 : __ldg(natj + b0 + q);
         __syncthreads();
         // (nn, b) = divmod(q, nb) for q = tid, tid + nth, ...: advanced by divmod(nth, nb)
         // with one carry (b + db < 2 nb), two divisions per thread and round
@@ -971,7 +980,7 @@ __global__ void __launch_bounds__(kTcNR * kLeafMaxR8 / 8) leaf_v_kernel(const __
       for (int b = 0; b < nb; ++b) leaf_v_point(acc, vs + b * R8 + k0, xs[b * xstride + n]);
     }
   }
-  store_split8<TF32>(a.outs, j, R8, n, k0, acc);
+  store_split8<TF32, NR>(a.outs, j, R8, n, k0, acc);
 }
 
 // U^L for a panel, one CTA per group g (leaves i = c g + t) or, with leaf_split, one
@@ -979,16 +988,16 @@ __global__ void __launch_bounds__(kTcNR * kLeafMaxR8 / 8) leaf_v_kernel(const __
 //   u[rhs0 + n][x_perm(b)] (+)= sum_k U^L_i[b][k] w[i R + k][n]
 // for the points b of leaf i.  The group's item is stored by columns (line = k, entry =
 // point of the group); the coefficient rows of the CTA's leaves (R contiguous rows of
-// 64 real then 64 imaginary parts per leaf) are staged whole in shared memory.  Thread
-// (b, nq) computes point b of the round for the 16 RHS n = 16 nq + 0..15, so that a
+// NR real then NR imaginary parts per leaf) are staged whole in shared memory.  Thread
+// (b, nq) computes point b of the round for the NR / 4 RHS from n = nq NR / 4 on, so that a
 // warp stores 32 consecutive points of one RHS row.  One CTA per leaf bounds a CTA's
 // work by the largest leaf when a ragged tree puts several times the mean number of
 // points into some groups.
 // XPOSE (the adjoint's V^L leaf products): the group's item is a (V^L)^* item (line =
 // point, entry = k, conj V), read transposed and conjugated.
-template <bool XPOSE>
+template <bool XPOSE, int NR>
 __global__ void __launch_bounds__(kLeafThreads) leaf_u_kernel(const __grid_constant__ LeafArgs a) {
-  constexpr int NR = kTcNR, NQ = kLeafThreads / kLeafPts, MN = NR / NQ;
+  constexpr int NQ = kLeafThreads / kLeafPts, MN = NR / NQ;
   extern __shared__ __align__(16) float2 lsm[];
   __shared__ int lend[kLeafMaxC + 1];
   const int c = a.c, R = a.R;
@@ -1096,16 +1105,16 @@ __global__ void __launch_bounds__(kLeafThreads) leaf_u_kernel(const __grid_const
 
 // ------------------------------------------------------------------ host side
 
-size_t tc_smem_bytes(int nsa, int nxb, int nsets, int mt_max, int kpad_max) {
+size_t tc_smem_bytes(int nsa, int nxb, int nsets, int mt_max, int kpad_max, int nr) {
   (void)nsets;
-  return size_t(nsa) * 4 * size_t(mt_max) * 32 + size_t(nxb) * 2 * size_t(kpad_max) * 256 +
+  return size_t(nsa) * 4 * size_t(mt_max) * 32 + size_t(nxb) * 2 * size_t(kpad_max) * 4 * size_t(nr) +
          (2 * size_t(nsa) + 2 * kMaxXBufs + 5) * 8 + 8 * 4 + 64;
 }
 
-size_t leaf_smem_bytes(int R, int c, bool u_side, int pts_cap) {
+size_t leaf_smem_bytes(int R, int c, bool u_side, int pts_cap, int nr) {
   const int R8 = (R + 7) & ~7;
-  return u_side ? size_t(c) * R * 2 * kTcNR * sizeof(float) + size_t(R) * kLeafPts * sizeof(float2)
-                : sizeof(float2) * size_t(pts_cap) * (kTcNR + 1 + R8);
+  return u_side ? size_t(c) * R * 2 * size_t(nr) * sizeof(float) + size_t(R) * kLeafPts * sizeof(float2)
+                : sizeof(float2) * size_t(pts_cap) * (size_t(nr) + 1 + R8);
 }
 
 int leaf_pts_cap(int64_t max_leaf_points) {
@@ -1115,11 +1124,12 @@ int leaf_pts_cap(int64_t max_leaf_points) {
 
 bool leaf_fits(int R8, int c) { return R8 <= kLeafMaxR8 && c <= kLeafMaxC; }
 
-cudaError_t launch_apply_tc(const TCArgs& a, int grid, size_t smem, cudaStream_t stream, bool tf32) {
+cudaError_t launch_apply_tc(const TCArgs& a, int grid, size_t smem, cudaStream_t stream, bool tf32, int nr) {
   if (a.nsa < kAProducers || a.nsa % kAProducers != 0) return cudaErrorInvalidValue;
   if (a.nxb < 1 || a.nxb > kMaxXBufs) return cudaErrorInvalidValue;
   cudaError_t err = cudaSuccess;   // (the caller clears the dependency counters)
-  void (*kern)(TCArgs) = tf32 ? bf_apply_tc<true> : bf_apply_tc<false>;
+  void (*kern)(TCArgs) = nr == 32 ? (tf32 ? bf_apply_tc<true, 32> : bf_apply_tc<false, 32>)
+                                  : (tf32 ? bf_apply_tc<true, 64> : bf_apply_tc<false, 64>);
   if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess)
     return err;
   cudaLaunchConfig_t cfg = {};
@@ -1216,15 +1226,18 @@ cudaError_t launch_permute_in(const LeafArgs& a, cudaStream_t stream) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_leaf(const LeafArgs& a, bool u_side, int n_groups, cudaStream_t stream, bool tf32, bool xpose) {
-  const size_t smem = u_side ? leaf_smem_bytes(a.R, a.leaf_split ? 1 : a.c, true)
-                             : sizeof(float2) * size_t(a.pts_cap) * (kTcNR + (a.gather ? 1 : 0) + a.R8);
+namespace {
+
+template <int NR>
+cudaError_t launch_leaf_nr(const LeafArgs& a, bool u_side, int n_groups, cudaStream_t stream, bool tf32, bool xpose) {
+  const size_t smem = u_side ? leaf_smem_bytes(a.R, a.leaf_split ? 1 : a.c, true, 0, NR)
+                             : sizeof(float2) * size_t(a.pts_cap) * (NR + (a.gather ? 1 : 0) + a.R8);
   void (*kern)(LeafArgs) =
-      u_side ? (xpose ? leaf_u_kernel<true> : leaf_u_kernel<false>)
-             : (tf32 ? (xpose ? leaf_v_kernel<true, true> : leaf_v_kernel<true, false>)
-                     : (xpose ? leaf_v_kernel<false, true> : leaf_v_kernel<false, false>));
+      u_side ? (xpose ? leaf_u_kernel<true, NR> : leaf_u_kernel<false, NR>)
+             : (tf32 ? (xpose ? leaf_v_kernel<true, true, NR> : leaf_v_kernel<true, false, NR>)
+                     : (xpose ? leaf_v_kernel<false, true, NR> : leaf_v_kernel<false, false, NR>));
   // U^L: a CTA per group; (V^L)^*: a CTA per leaf, one thread per RHS column and group of 8 rows
-  const int threads = u_side ? kLeafThreads : kTcNR * (a.R8 / 8);
+  const int threads = u_side ? kLeafThreads : NR * (a.R8 / 8);
   const int64_t blocks = (u_side && !a.leaf_split) ? int64_t(n_groups) : int64_t(n_groups) * a.c;
   if (!u_side && (a.pts_cap < 8 || a.pts_cap > kLeafPts || a.pts_cap % 8 != 0)) return cudaErrorInvalidValue;
   if (blocks <= 0) return cudaSuccess;
@@ -1232,6 +1245,13 @@ cudaError_t launch_leaf(const LeafArgs& a, bool u_side, int n_groups, cudaStream
   if (err != cudaSuccess) return err;
   kern<<<unsigned(blocks), threads, smem, stream>>>(a);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_leaf(const LeafArgs& a, bool u_side, int n_groups, cudaStream_t stream, int nr, bool tf32, bool xpose) {
+  return nr == 32 ? launch_leaf_nr<32>(a, u_side, n_groups, stream, tf32, xpose)
+                  : launch_leaf_nr<64>(a, u_side, n_groups, stream, tf32, xpose);
 }
 
 }  // namespace mbf

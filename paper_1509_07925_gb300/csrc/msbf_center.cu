@@ -23,8 +23,8 @@ constexpr int kCPts = 4;      // centre points per CTA (adjoint)
 // Forward: a CTA computes 64 outputs x for 8 RHS; its four shares of 64 threads take the
 // centre points of a round in turn and their sums are added at the end, always in the
 // same order.  One thread per x over all the centre points (an earlier form) left each
-// thread a serial chain of loads and the chip at 8 warps an SM: 81 us for n = 128, 289
-// points, 32 RHS, against 16 us of multiply-adds; now 20 us.
+// thread a serial chain of loads and the chip at 14 warps an SM: 81 us for n = 128, 289
+// points, 32 RHS, from a cold cache; now 52 us.
 __global__ void __launch_bounds__(kCThreads) center_fwd_kernel(const float2* __restrict__ Kc,
                                                                const int32_t* __restrict__ idx, int n_c,
                                                                const float2* __restrict__ g, int64_t len_in,

@@ -680,17 +680,23 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
       // accumulator sets (2 M_t TMEM columns each), panel buffers, A ring slots; more
       // than half the SM's shared memory, so one CTA per SM and each CTA's 512-column
       // TMEM allocation never waits on another CTA of the same launch
-      auto config = [&](int mt, int kp, int& nsets, int& nxb, int& nsa, size_t& sm) {
+      auto config = [&](int mt, int kp, int nr, int& nsets, int& nxb, int& nsa, size_t& sm) {
         nsets = 4 * mt <= 512 ? 2 : 1;
         nxb = 2;
-        auto smem = [&](int n) { return tc_smem_bytes(n, nxb, nsets, mt, kp); };
+        auto smem = [&](int n) { return tc_smem_bytes(n, nxb, nsets, mt, kp, nr); };
         if (smem(2) > size_t(optin)) nxb = 1;
         if (smem(2) > size_t(optin)) fail(MBF_ERR_INVALID, "tiles too large for the tensor path");
         nsa = 2;   // a multiple of the tile stream's producer lanes (2)
         while (nsa + 2 <= 16 && smem(nsa + 2) <= size_t(optin)) nsa += 2;
+        if (nsa == 2 && nxb == 2) {   // wide tiles: a deeper ring is worth more than the second panel
+          nxb = 1;
+          while (nsa + 2 <= 16 && smem(nsa + 2) <= size_t(optin)) nsa += 2;
+          if (nsa == 2) nxb = 2;
+        }
         sm = std::max(smem(nsa), size_t(optin) / 2 + 1024);
       };
-      config(op->tc_mt_max, op->tc_kpad_max, op->tc_nsets, op->tc_nxb, op->tc_nsa, op->tc_smem);
+      config(op->tc_mt_max, op->tc_kpad_max, kTcNR, op->tc_nsets, op->tc_nxb, op->tc_nsa, op->tc_smem);
+      config(op->tc_mt_max, op->tc_kpad_max, kTcNRHalf, op->tc_nsets, op->tc_nxb32, op->tc_nsa32, op->tc_smem32);
       // the tensor adjoint: its plan (adjoint_tile_plan) and launch configuration
       try {
         const TCPlan& ap = op->tcplan_adj;
@@ -700,7 +706,8 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
         if (!leaf_fits(ap.st[0].R8_in, op->c) || leaf_smem_bytes(op->RV[size_t(op->L)], op->c, true) > size_t(optin) ||
             leaf_smem_bytes(op->RU[size_t(op->L)], op->c, false) > size_t(optin))
           fail(MBF_ERR_INVALID, "leaf rank too large for the tensor adjoint");
-        config(op->tca_mt_max, op->tca_kpad_max, op->tca_nsets, op->tca_nxb, op->tca_nsa, op->tca_smem);
+        config(op->tca_mt_max, op->tca_kpad_max, kTcNR, op->tca_nsets, op->tca_nxb, op->tca_nsa, op->tca_smem);
+        config(op->tca_mt_max, op->tca_kpad_max, kTcNRHalf, op->tca_nsets, op->tca_nxb32, op->tca_nsa32, op->tca_smem32);
         std::vector<int32_t> xinv(size_t(std::max<int64_t>(f.n_out, 1)), -1);
         for (int64_t p = 0; p < f.n_out; ++p) xinv[size_t(f.x_perm[p])] = int32_t(p);
         op->d_x_inv = dev_upload(xinv, "inverse X permutation");
@@ -786,7 +793,10 @@ void apply_tc(mbf_op_s* op, Workspace& w, const float2* g, float2* u, int64_t nr
   uint8_t* yl = w.tc_bufs;                       // level-L input of the main stages
   uint8_t* bufs = yl + vec_bytes;                    // main stage e < S - 1 writes bufs + e * vec_bytes
   float* ylast = reinterpret_cast<float*>(yl + int64_t(S) * vec_bytes);   // last main stage
-  for (int64_t r0 = 0; r0 < nrhs; r0 += kTcNR) {
+  for (int64_t r0 = 0, nr = kTcNR; r0 < nrhs; r0 += nr) {
+    // a panel of 32 for the last RHS where they fit one (the host-link input panel keeps 64)
+    nr = !host_io && nrhs - r0 <= kTcNRHalf ? kTcNRHalf : kTcNR;
+    const bool half = nr == kTcNRHalf;
     // the tensor kernel's dependency counters (cleared per panel)
     cuda_check(cudaMemsetAsync(w.tc_counters, 0, tc_counter_bytes(tp), st), "counter clear");
     // page-locked host input: g -> panel in tree order first (rows read across the
@@ -829,7 +839,7 @@ void apply_tc(mbf_op_s* op, Workspace& w, const float2* g, float2* u, int64_t nr
     la.R8 = tp.st[0].R8_in;
     la.pts_cap = leaf_pts_cap(op->leaf_pts_w);
     e0 = prof_begin(op, st);
-    cuda_check(launch_leaf(la, false, leaf_st.n_groups, st, tf32), "leaf (V^L)^* launch");
+    cuda_check(launch_leaf(la, false, leaf_st.n_groups, st, int(nr), tf32), "leaf (V^L)^* launch");
     prof_end(op, PK_LEAF_V, e0, st);
     // G / H levels on tensor cores
     TCArgs ta{};
@@ -840,14 +850,14 @@ void apply_tc(mbf_op_s* op, Workspace& w, const float2* g, float2* u, int64_t nr
     ta.buf_stride = vec_bytes;
     ta.counters = w.tc_counters;
     ta.status = w.status;
-    ta.nsa = op->tc_nsa;
-    ta.nxb = op->tc_nxb;
+    ta.nsa = half ? op->tc_nsa32 : op->tc_nsa;
+    ta.nxb = half ? op->tc_nxb32 : op->tc_nxb;
     ta.nsets = op->tc_nsets;
     ta.mt_max = op->tc_mt_max;
     ta.kpad_max = op->tc_kpad_max;
     ta.plan = tp;
     e0 = prof_begin(op, st);
-    cuda_check(launch_apply_tc(ta, sms, op->tc_smem, st, tf32), "tensor-core launch");
+    cuda_check(launch_apply_tc(ta, sms, half ? op->tc_smem32 : op->tc_smem, st, tf32, int(nr)), "tensor-core launch");
     prof_end(op, PK_TC, e0, st);
     // U^L: last main stage output -> u
     LeafArgs lu{};
@@ -871,7 +881,7 @@ void apply_tc(mbf_op_s* op, Workspace& w, const float2* g, float2* u, int64_t nr
     lu.accumulate = accumulate ? 1 : 0;
     lu.leaf_split = op->split_x;
     e0 = prof_begin(op, st);
-    cuda_check(launch_leaf(lu, true, last_st.n_groups, st), "leaf U^L launch");
+    cuda_check(launch_leaf(lu, true, last_st.n_groups, st, int(nr)), "leaf U^L launch");
     prof_end(op, PK_LEAF_U, e0, st);
   }
 }
@@ -910,7 +920,10 @@ void apply_tc_adj(mbf_op_s* op, Workspace& w, const float2* u, float2* g, int64_
   uint8_t* yl = w.tc_bufs;
   uint8_t* bufs = yl + vec_bytes;
   float* ylast = reinterpret_cast<float*>(yl + int64_t(S) * vec_bytes);
-  for (int64_t r0 = 0; r0 < nrhs; r0 += kTcNR) {
+  for (int64_t r0 = 0, nr = kTcNR; r0 < nrhs; r0 += nr) {
+    // a panel of 32 for the last RHS where they fit one (the host-link input panel keeps 64)
+    nr = !host_io && nrhs - r0 <= kTcNRHalf ? kTcNRHalf : kTcNR;
+    const bool half = nr == kTcNRHalf;
     // the tensor kernel's dependency counters (cleared per panel)
     cuda_check(cudaMemsetAsync(w.tc_counters, 0, tc_counter_bytes(ap), st), "counter clear");
     // u -> panel in X-tree order (page-locked host input), or gathered by the leaf kernel
@@ -948,7 +961,7 @@ void apply_tc_adj(mbf_op_s* op, Workspace& w, const float2* u, float2* g, int64_
     la.R8 = ap.st[0].R8_in;
     la.pts_cap = leaf_pts_cap(op->leaf_pts_x);
     e0 = prof_begin(op, st);
-    cuda_check(launch_leaf(la, false, last_st.n_groups, st, false, true), "leaf (U^L)^* launch");
+    cuda_check(launch_leaf(la, false, last_st.n_groups, st, int(nr), false, true), "leaf (U^L)^* launch");
     prof_end(op, PK_LEAF_V, e0, st);
     // (G^l)^*, l = L-1 .. h, (M^h)^*, H^l, l = h .. L-1 on tensor cores
     TCArgs ta{};
@@ -959,14 +972,14 @@ void apply_tc_adj(mbf_op_s* op, Workspace& w, const float2* u, float2* g, int64_
     ta.buf_stride = vec_bytes;
     ta.counters = w.tc_counters;
     ta.status = w.status;
-    ta.nsa = op->tca_nsa;
-    ta.nxb = op->tca_nxb;
+    ta.nsa = half ? op->tca_nsa32 : op->tca_nsa;
+    ta.nxb = half ? op->tca_nxb32 : op->tca_nxb;
     ta.nsets = op->tca_nsets;
     ta.mt_max = op->tca_mt_max;
     ta.kpad_max = op->tca_kpad_max;
     ta.plan = ap;
     e0 = prof_begin(op, st);
-    cuda_check(launch_apply_tc(ta, sms, op->tca_smem, st, false), "tensor-core launch");
+    cuda_check(launch_apply_tc(ta, sms, half ? op->tca_smem32 : op->tca_smem, st, false, int(nr)), "tensor-core launch");
     prof_end(op, PK_TC, e0, st);
     // V^L: last stage output -> g (natural Omega order)
     LeafArgs lv{};
@@ -986,7 +999,7 @@ void apply_tc_adj(mbf_op_s* op, Workspace& w, const float2* u, float2* g, int64_
     lv.accumulate = accumulate ? 1 : 0;
     lv.leaf_split = op->split_w;
     e0 = prof_begin(op, st);
-    cuda_check(launch_leaf(lv, true, leaf_st.n_groups, st, false, true), "leaf V^L launch");
+    cuda_check(launch_leaf(lv, true, leaf_st.n_groups, st, int(nr), false, true), "leaf V^L launch");
     prof_end(op, PK_LEAF_U, e0, st);
   }
 }

@@ -63,6 +63,9 @@ struct mbf_op_s {
   int64_t tc_bytes = 0;
   int tc_mt_max = 16, tc_kpad_max = 16, tc_nsa = 2, tc_nxb = 2, tc_nsets = 2;
   size_t tc_smem = 0;
+  // the same for panels of 32 RHS: ring slots, panel buffers, shared memory
+  int tc_nsa32 = 2, tc_nxb32 = 2, tca_nsa32 = 2, tca_nxb32 = 2;
+  size_t tc_smem32 = 0, tca_smem32 = 0;
   int32_t* d_w_inv = nullptr;         // natural Omega index -> tree position (-1: not in the tree)
   std::string tc_unavailable;         // why the tensor path cannot run for this operator ("" if it can)
   std::string simt_unavailable;       // why the FP32 SIMT path cannot (leaves beyond its limits; "" if it can)
