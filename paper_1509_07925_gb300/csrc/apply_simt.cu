@@ -992,32 +992,43 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
                 }
               }
             } else {
-              // the warp's sums go to its share of `red`: [share][RHS][entry]
+              // the warp's sums go to its share of `red`, [share][entry][RHS] in float4 units (two
+              // RHS), unit u of entry e at u ^ swz(e): a quarter warp's writes (8 entries, one
+              // unit) and its reads (consecutive units) both touch every bank once
+              constexpr int U = NR / 2 > 0 ? NR / 2 : 1;
+              const auto swz = [](int ee) { return NR == 8 ? (ee >> 1) & 3 : (ee >> 2) & 1; };
+              float4* red4 = reinterpret_cast<float4*>(red);
 #pragma unroll
               for (int q = 0; q < 4; ++q) {
                 const int ee = ea + lane + 32 * q;
                 if (q < je && ee < min(tot, ea + part))
 #pragma unroll
-                  for (int r = 0; r < NR; ++r) red[(ks * NRB + r) * tot + ee] = acc[q][r];
+                  for (int u = 0; u < U; ++u)
+                    red4[(ks * tot + ee) * U + (u ^ swz(ee))] =
+                        make_float4(acc[q][(2 * u) % NR].x, acc[q][(2 * u) % NR].y, acc[q][(2 * u + 1) % NR].x,
+                                    acc[q][(2 * u + 1) % NR].y);
               }
               cons_sync<W>();
               if (ok)
-                by_rhs(tot, [&](int q, int r) {
-                  float2 v = red[r * tot + q];
+                for (int q = tid; q < tot * U; q += W * 32) {
+                  const int ee = q / U, u = q % U, at = ee * U + (u ^ swz(ee));
+                  float4 v = red4[at];
 #pragma unroll
                   for (int k = 1; k < W; ++k)
                     if (k < 1 << lks) {
-                      const float2 w = red[(k * NRB + r) * tot + q];
+                      const float4 w = red4[k * tot * U + at];
                       v.x += w.x;
                       v.y += w.y;
+                      v.z += w.z;
+                      v.w += w.w;
                     }
                   if (out_pat == PAT_LEAF) {
-                    ybuf[q * NRB + r] = v;
+                    *reinterpret_cast<float4*>(ybuf + ee * NRB + 2 * u) = v;
                   } else {
-                    const int t = seg_of(q, Rout, c);
-                    dst[int64_t(m.out.base + t * m.out.step + q - t * Rout) * NRB + r] = v;
+                    const int t = seg_of(ee, Rout, c);
+                    *reinterpret_cast<float4*>(dst + int64_t(m.out.base + t * m.out.step + ee - t * Rout) * NRB + 2 * u) = v;
                   }
-                });
+                }
             }
             if (out_pat == PAT_LEAF) {
               // U^L of the block's outputs (ybuf): lines are the columns, entries the group's points,
