@@ -108,7 +108,8 @@ struct LeafArgs {
   int32_t R8, item_stride;
   int32_t accumulate;       // U^L: 1 adds into u
   int32_t pts_cap;          // (V^L)^*: points staged per round (leaf_pts_cap of the largest leaf)
-  int32_t leaf_split;       // U^L side: 1 = one CTA per leaf (ragged trees), 0 = one per group
+  int32_t leaf_split;       // U^L side: 1 = one CTA per leaf (ragged trees, few groups), 0 = one per group
+  int32_t small_leaves;     // U^L side, leaf_split: rounds of 16 points instead of 64
   int32_t gather;           // (V^L)^* side: 1 = vec is [nrhs][len_vec] in natural order, read through
                             // nat; 0 = the tree-ordered panel
   int32_t nat_stride;       // (V^L)^* gather: entries per leaf in nat

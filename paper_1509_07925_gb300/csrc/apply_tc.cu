@@ -936,27 +936,20 @@ __global__ void __launch_bounds__(NR * kLeafMaxR8 / 8) leaf_v_kernel(const __gri
       } else {
         for (int q = tid; q < nb * (NR / 2); q += nth) cp_async16(sa(xs) + uint32_t(q) * 16u, src + 2 * q);
       }
-      const int lpc = it.lpc;
-      for (int b1 = bq; b1 < nb; b1 += 8 * bstep) {             // 8 loads in flight per thread
-        float2 v[8];
-        // forward: line pt of the item, as (chunk, line in chunk), advanced by bstep per u
-        int ci = 0, li = 0;
-        if (!XPOSE) {
-          const int line = p0 - pg + b0 + b1;
-          ci = line / lpc;
-          li = line - ci * lpc;
-        }
+      // entry kq of points b1, b1 + bstep, ...: the item's line is the point (chunk ci, line li
+      // within it, advanced by bstep) or, XPOSE, the column kq (fixed)
+      const int lpc = it.lpc, line0 = XPOSE ? min(kq, R - 1) : p0 - pg + b0 + bq;
+      int ci = line0 / lpc, li = line0 - ci * lpc;
+      constexpr int F = XPOSE ? 4 : 8;   // (4 transposed: 32.3 -> 29.6 us of the adjoint; forward 46.3, with 4 49.6)
+      for (int b1 = bq; b1 < nb; b1 += F * bstep) {             // F loads in flight per thread
+        float2 v[F];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int b = b1 + u * bstep, pt = p0 - pg + b0 + b;
+        for (int u = 0; u < F; ++u) {
+          const int b = b1 + u * bstep;
           v[u] = make_float2(0.f, 0.f);
           if (b < nb && kq < R) {
-            if (XPOSE) {
-              const float2 e = item_entry(ibase, it, kq, pt);
-              v[u] = make_float2(e.x, -e.y);
-            } else {
-              v[u] = item_entry_cl(ibase, it, ci, li, kq);
-            }
+            const float2 e = item_entry_cl(ibase, it, ci, li, XPOSE ? p0 - pg + b0 + b : kq);
+            v[u] = XPOSE ? make_float2(e.x, -e.y) : e;
           }
           if (!XPOSE) {
             li += bstep;
@@ -967,7 +960,7 @@ __global__ void __launch_bounds__(NR * kLeafMaxR8 / 8) leaf_v_kernel(const __gri
           }
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < F; ++u)
           if (b1 + u * bstep < nb) vs[(b1 + u * bstep) * R8 + kq] = v[u];
       }
       cp_async_wait_all();
@@ -995,9 +988,12 @@ __global__ void __launch_bounds__(NR * kLeafMaxR8 / 8) leaf_v_kernel(const __gri
 // points into some groups.
 // XPOSE (the adjoint's V^L leaf products): the group's item is a (V^L)^* item (line =
 // point, entry = k, conj V), read transposed and conjugated.
-template <bool XPOSE, int NR>
+// PT: points of a round (and threads along the points).  64 where a CTA has that many;
+// 16 for a CTA per small leaf, where 48 of 64 such threads would idle: the polar Omega
+// side (mean 16 points a leaf) of the adjoint, n = 256, 64 RHS: 65 us with 64, 56 with 16.
+template <bool XPOSE, int NR, int PT>
 __global__ void __launch_bounds__(kLeafThreads) leaf_u_kernel(const __grid_constant__ LeafArgs a) {
-  constexpr int NQ = kLeafThreads / kLeafPts, MN = NR / NQ;
+  constexpr int NQ = kLeafThreads / PT, MN = NR / NQ, MV = MN < 4 ? MN : 4;
   extern __shared__ __align__(16) float2 lsm[];
   __shared__ int lend[kLeafMaxC + 1];
   const int c = a.c, R = a.R;
@@ -1011,7 +1007,7 @@ __global__ void __launch_bounds__(kLeafThreads) leaf_u_kernel(const __grid_const
   const Item it = a.items[a.item_base + int64_t(g) * a.item_stride];
   const uint8_t* ibase = a.arena + size_t(it.off128) * 128;
   float* ws = reinterpret_cast<float*>(lsm);                        // [nl R][2 NR]
-  float2* us = reinterpret_cast<float2*>(ws + size_t(nl) * R * 2 * NR);   // [R][kLeafPts]
+  float2* us = reinterpret_cast<float2*>(ws + size_t(nl) * R * 2 * NR);   // [R][PT]
   const float* rows_g = a.wl + (int64_t(c) * g + t0) * R * 2 * NR;     // the CTA's leaves' rows
   {
     const float4* src = reinterpret_cast<const float4*>(rows_g);
@@ -1027,38 +1023,66 @@ __global__ void __launch_bounds__(kLeafThreads) leaf_u_kernel(const __grid_const
         if (q0 + u * kLeafThreads < nq4) dst[q0 + u * kLeafThreads] = v[u];
     }
   }
-  const int bb = tid % kLeafPts, nq = tid / kLeafPts;
+  const int bb = tid % PT, nq = tid / PT;
   __syncthreads();
   {   // the rows are read by this CTA alone and never again: drop them from L2
     using tc::l2_discard;
     const char* rows = reinterpret_cast<const char*>(rows_g);
     for (int q = tid; q < nl * R * (2 * NR * int(sizeof(float)) / 128); q += kLeafThreads) l2_discard(rows + 128 * q);
   }
-  for (int b0 = 0; b0 < np; b0 += kLeafPts) {
-    const int nb = min(kLeafPts, np - b0);
+  for (int b0 = 0; b0 < np; b0 += PT) {
+    const int nb = min(PT, np - b0);
     if (b0 > 0) __syncthreads();
-    for (int q0 = tid; q0 < R * nb; q0 += 8 * kLeafThreads) {   // 8 loads in flight per thread
-      float2 v[8];
+    // (PT = 16) entries k = nq, nq + NQ, ... of point bb: the item's line is the point (XPOSE, fixed) or
+    // the column k (chunk ci, line li within it, advanced by NQ), so one division a round
+    if (PT == 16 && bb < nb) {
+      const int lpc = it.lpc, line0 = XPOSE ? pb + b0 + bb : nq;
+      int ci = line0 / lpc, li = line0 - ci * lpc;
+      for (int k0 = nq; k0 < R; k0 += 8 * NQ) {                 // 8 loads in flight per thread
+        float2 v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int q = q0 + u * kLeafThreads, k = q / nb, b = q - k * nb;
-        if (q < R * nb) {
-          if (XPOSE) {
-            const float2 e = item_entry(ibase, it, pb + b0 + b, k);
-            v[u] = make_float2(e.x, -e.y);
-          } else {
-            v[u] = item_entry(ibase, it, k, pb + b0 + b);
+        for (int u = 0; u < 8; ++u) {
+          const int k = k0 + u * NQ;
+          if (k < R) {
+            const float2 e = item_entry_cl(ibase, it, ci, li, XPOSE ? k : pb + b0 + bb);
+            v[u] = XPOSE ? make_float2(e.x, -e.y) : e;
+            if (!XPOSE) {
+              li += NQ;
+              while (li >= lpc) {
+                li -= lpc;
+                ++ci;
+              }
+            }
           }
-        } else {
-          v[u] = make_float2(0.f, 0.f);
         }
-      }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int q = q0 + u * kLeafThreads, k = q / nb, b = q - k * nb;
-        if (q < R * nb) us[k * kLeafPts + b] = v[u];
+        for (int u = 0; u < 8; ++u)
+          if (k0 + u * NQ < R) us[(k0 + u * NQ) * PT + bb] = v[u];
       }
     }
+    if (PT != 16)
+      for (int q0 = tid; q0 < R * nb; q0 += 8 * kLeafThreads) {   // 8 loads in flight per thread
+        float2 v[8];
+  #pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int q = q0 + u * kLeafThreads, k = q / nb, b = q - k * nb;
+          if (q < R * nb) {
+            if (XPOSE) {
+              const float2 e = item_entry(ibase, it, pb + b0 + b, k);
+              v[u] = make_float2(e.x, -e.y);
+            } else {
+              v[u] = item_entry(ibase, it, k, pb + b0 + b);
+            }
+          } else {
+            v[u] = make_float2(0.f, 0.f);
+          }
+        }
+  #pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int q = q0 + u * kLeafThreads, k = q / nb, b = q - k * nb;
+          if (q < R * nb) us[k * PT + b] = v[u];
+        }
+      }
     __syncthreads();
     if (bb < nb) {
       const int p = pb + b0 + bb;                 // group-relative point
@@ -1069,16 +1093,25 @@ __global__ void __launch_bounds__(kLeafThreads) leaf_u_kernel(const __grid_const
 #pragma unroll
       for (int j = 0; j < MN; ++j) acc[j] = make_float2(0.f, 0.f);
       for (int k = 0; k < R; ++k) {
-        const float2 uv = us[k * kLeafPts + bb];
+        const float2 uv = us[k * PT + bb];
         const float* wk = wr + k * 2 * NR;
 #pragma unroll
-        for (int j4 = 0; j4 < MN / 4; ++j4) {
-          const float4 wre = *reinterpret_cast<const float4*>(wk + 4 * j4);
-          const float4 wim = *reinterpret_cast<const float4*>(wk + NR + 4 * j4);
-          const float re[4] = {wre.x, wre.y, wre.z, wre.w}, im[4] = {wim.x, wim.y, wim.z, wim.w};
+        for (int jv = 0; jv < MN / MV; ++jv) {
+          float re[MV], im[MV];
+          if constexpr (MV == 4) {
+            const float4 wre = *reinterpret_cast<const float4*>(wk + 4 * jv);
+            const float4 wim = *reinterpret_cast<const float4*>(wk + NR + 4 * jv);
+            re[0] = wre.x, re[1] = wre.y, re[2] = wre.z, re[3] = wre.w;
+            im[0] = wim.x, im[1] = wim.y, im[2] = wim.z, im[3] = wim.w;
+          } else {
+            const float2 wre = *reinterpret_cast<const float2*>(wk + 2 * jv);
+            const float2 wim = *reinterpret_cast<const float2*>(wk + NR + 2 * jv);
+            re[0] = wre.x, re[1] = wre.y;
+            im[0] = wim.x, im[1] = wim.y;
+          }
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            float2& o = acc[4 * j4 + j];
+          for (int j = 0; j < MV; ++j) {
+            float2& o = acc[MV * jv + j];
             o.x = fmaf(uv.x, re[j], fmaf(-uv.y, im[j], o.x));
             o.y = fmaf(uv.x, im[j], fmaf(uv.y, re[j], o.y));
           }
@@ -1233,7 +1266,8 @@ cudaError_t launch_leaf_nr(const LeafArgs& a, bool u_side, int n_groups, cudaStr
   const size_t smem = u_side ? leaf_smem_bytes(a.R, a.leaf_split ? 1 : a.c, true, 0, NR)
                              : sizeof(float2) * size_t(a.pts_cap) * (NR + (a.gather ? 1 : 0) + a.R8);
   void (*kern)(LeafArgs) =
-      u_side ? (xpose ? leaf_u_kernel<true, NR> : leaf_u_kernel<false, NR>)
+      u_side ? (a.small_leaves ? (xpose ? leaf_u_kernel<true, NR, 16> : leaf_u_kernel<false, NR, 16>)
+                               : (xpose ? leaf_u_kernel<true, NR, kLeafPts> : leaf_u_kernel<false, NR, kLeafPts>))
              : (tf32 ? (xpose ? leaf_v_kernel<true, true, NR> : leaf_v_kernel<true, false, NR>)
                      : (xpose ? leaf_v_kernel<false, true, NR> : leaf_v_kernel<false, false, NR>));
   // U^L: a CTA per group; (V^L)^*: a CTA per leaf, one thread per RHS column and group of 8 rows

@@ -640,6 +640,14 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
     };
     op->split_x = few || ragged(f.x_off) ? 1 : 0;
     op->split_w = few || ragged(f.w_off) ? 1 : 0;
+    // mean points of the leaves that have any
+    auto small = [&](const int64_t* off, int64_t n) {
+      int64_t ne = 0;
+      for (int64_t q = 0; q < nL; ++q) ne += off[q + 1] > off[q];
+      return n <= 24 * ne;
+    };
+    op->small_x = op->split_x && small(f.x_off, f.n_out) ? 1 : 0;
+    op->small_w = op->split_w && small(f.w_off, f.n_w) ? 1 : 0;
     op->d_x_perm = dev_upload(to32(f.x_perm, f.n_out), "x_perm");
     op->d_x_off = dev_upload(to32(f.x_off, nL + 1), "x_off");
     op->d_w_perm = dev_upload(to32(f.w_perm, std::max<int64_t>(f.n_w, 1)), "w_perm");
@@ -880,6 +888,7 @@ void apply_tc(mbf_op_s* op, Workspace& w, const float2* g, float2* u, int64_t nr
     lu.R = op->RU[size_t(op->L)];
     lu.accumulate = accumulate ? 1 : 0;
     lu.leaf_split = op->split_x;
+    lu.small_leaves = op->small_x;
     e0 = prof_begin(op, st);
     cuda_check(launch_leaf(lu, true, last_st.n_groups, st, int(nr)), "leaf U^L launch");
     prof_end(op, PK_LEAF_U, e0, st);
@@ -998,6 +1007,7 @@ void apply_tc_adj(mbf_op_s* op, Workspace& w, const float2* u, float2* g, int64_
     lv.R = op->RV[size_t(op->L)];
     lv.accumulate = accumulate ? 1 : 0;
     lv.leaf_split = op->split_w;
+    lv.small_leaves = op->small_w;
     e0 = prof_begin(op, st);
     cuda_check(launch_leaf(lv, true, leaf_st.n_groups, st, int(nr), false, true), "leaf V^L launch");
     prof_end(op, PK_LEAF_U, e0, st);

@@ -49,7 +49,8 @@ struct mbf_op_s {
   // largest leaf rounded up to 8: the leaf kernels' gathers need no offset load first
   int32_t *d_x_nat = nullptr, *d_w_nat = nullptr;
   int32_t x_nat_stride = 0, w_nat_stride = 0;
-  int32_t split_x = 0, split_w = 0;         // U^L-side leaf kernels: one CTA per leaf (ragged tree)
+  int32_t split_x = 0, split_w = 0;         // U^L-side leaf kernels: one CTA per leaf (ragged tree, few groups)
+  int32_t small_x = 0, small_w = 0;         // and rounds of 16 points (leaves of at most 24 on average)
   mbf::Workspace ws;                // the scratch of the operator's own applies
   // SIMT kernel: its launch shapes by RHS per pass (1, 2, 4, 8); xcap: most entries of a
   // block side or points of a leaf group
