@@ -30,7 +30,13 @@ struct ApplyArgs {
   int64_t in_len, out_len;
   float2* bufs;            // stage e < S - 1 writes bufs + e * buf_stride ([pos][NRB]); stage e+1 reads it
   int64_t buf_stride;
-  unsigned int* counters;  // [stage][group]: input segments written so far (zeroed per launch)
+  // [stage][group]: input segments written so far.  With ctl, two sets of them: a launch
+  // counts in set ctl[0] & 1 and clears the other one for the next launch, so that no
+  // memset precedes it (the last CTA to finish, counted in ctl[1], flips ctl[0]; the state
+  // lives on the device, so a captured launch may be replayed).  Without, one set, cleared by
+  // launch_apply_simt.
+  unsigned int* counters;
+  unsigned int* ctl;
   int* status;             // 0 = ok; nonzero = a device wait ran out of time (sticky)
   int32_t nrhs, rhs0;      // this launch applies RHS rhs0 .. min(nrhs, rhs0 + NRB) - 1
   int32_t xcap;            // most entries of a block side or points of a leaf group (<= 256)
@@ -48,6 +54,35 @@ struct ApplyArgs {
   RowTable rows;
   Plan plan;
 };
+
+// Words before a workspace's counters: ctl[0], ctl[1] and padding.
+constexpr int kCtlWords = 64;
+// Bytes of a workspace's counters for a kernel that counts in `set_bytes`.
+MBF_HD size_t counters_alloc(size_t set_bytes) { return kCtlWords * sizeof(unsigned) + 2 * set_bytes; }
+
+#if defined(__CUDACC__)
+// The launch's counter set, of `words` counters.
+__device__ __forceinline__ unsigned* counter_set(unsigned* counters, const unsigned* ctl, unsigned words) {
+  return ctl && (__ldcg(ctl) & 1u) ? counters + words : counters;
+}
+// Clears this CTA's part of the other set (threads tid < nth of each CTA).
+__device__ __forceinline__ void clear_other_set(unsigned* counters, const unsigned* ctl, unsigned words, unsigned tid,
+                                                unsigned nth) {
+  if (!ctl) return;
+  unsigned* other = __ldcg(ctl) & 1u ? counters : counters + words;
+  for (unsigned i = blockIdx.x * nth + tid; i < words; i += gridDim.x * nth) other[i] = 0;
+}
+// By one thread of each CTA when all the CTA's counting is done: the last one flips the sets.
+__device__ __forceinline__ void finish_counters(unsigned* ctl) {
+  if (!ctl) return;
+  const unsigned epoch = __ldcg(ctl);
+  __threadfence();
+  if (atomicAdd(ctl + 1, 1u) == gridDim.x - 1) {
+    ctl[1] = 0;
+    ctl[0] = epoch ^ 1u;
+  }
+}
+#endif
 
 enum DeviceStatus : int {
   ST_OK = 0,
@@ -85,7 +120,8 @@ struct TCArgs {
   uint8_t* bufs;           // output of main stage e < S - 1: bufs + e * buf_stride (split blocks)
   float* y_out;            // output of the last main stage: row block * R + k, [re NR | im NR] floats
   int64_t buf_stride;      // bytes
-  unsigned* counters;      // [stage][group], zeroed per launch
+  unsigned* counters;      // [stage][group], two sets as in ApplyArgs
+  unsigned* ctl;
   int* status;
   int32_t nsa, nxb;        // A ring slots; panel buffers (1 or 2)
   int32_t nsets, mt_max;   // accumulator sets (1 or 2, 2 mt_max TMEM columns each); largest M_t

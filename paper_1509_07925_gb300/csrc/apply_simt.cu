@@ -459,6 +459,7 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
   const int grid = int(gridDim.x);
   const auto first_group = [&](int e) { return int((blockIdx.x + unsigned(e) * unsigned(a.rot)) % unsigned(grid)); };
   const auto stage_of = [&](int e) -> const Stage& { return plan.st[ADJ ? S - 1 - e : e]; };
+  const unsigned n_cnt = unsigned(S) * unsigned(plan.st[0].n_groups);   // (every stage has as many groups)
 
   if (warp == W + GA) {
     // ------------------------------------------------------------------ producer
@@ -555,11 +556,12 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
     // stored by then.
     unsigned j = 0, avail = 0;
     bool ok = true;
+    unsigned* counters = counter_set(a.counters, a.ctl, n_cnt);
     for (int e = 0; e + 1 < S && ok; ++e) {
       const Stage& st = stage_of(e);
       const Stage& nst = stage_of(e + 1);
       const int out_pat = ADJ ? st.in_pat : st.out_pat, next_in = ADJ ? nst.out_pat : nst.in_pat;
-      unsigned* cnt_out = a.counters + int64_t(e + 1) * nst.n_groups;
+      unsigned* cnt_out = counters + int64_t(e + 1) * nst.n_groups;
       for (int g = first_group(e); g < st.n_groups; g += grid, ++j) {
         if (j >= avail) {
           uint64_t t0 = 0;
@@ -592,6 +594,7 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
     GroupMeta& m = meta[gw];
     unsigned j = 0;
     bool ok = true;
+    const unsigned* counters = counter_set(a.counters, a.ctl, n_cnt);
     for (int e = 0; e < S && ok; ++e) {
       const Stage& st = stage_of(e);
       const int in_pat = ADJ ? st.out_pat : st.in_pat, out_pat = ADJ ? st.in_pat : st.out_pat;
@@ -600,7 +603,7 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
       const int32_t* lperm = leaf_w ? a.w_perm : a.x_perm;
       const int32_t* loff = leaf_w ? a.w_off : a.x_off;
       const float2* src = a.bufs + (e > 0 ? e - 1 : 0) * a.buf_stride;
-      const unsigned* cnt_in = a.counters + int64_t(e) * st.n_groups;
+      const unsigned* cnt_in = counters + int64_t(e) * st.n_groups;
       for (int g = first_group(e); g < st.n_groups && ok; g += grid, ++j) {
         if (int(j % GA) != gw) continue;
         if (!__all_sync(0xffffffffu, wait_bar(&xempty[gw], ((j / GA) & 1u) ^ 1u, a, abort, lim, ST_EMPTY_TIMEOUT))) {
@@ -751,6 +754,7 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
     // ------------------------------------------------------------------ consumers
     constexpr bool kVec = NRB <= 2;                  // lane mapping of the main blocks (forward)
     const int tid = threadIdx.x;
+    clear_other_set(a.counters, a.ctl, n_cnt, unsigned(tid), W * 32);
     const uint32_t ring_a = smem_addr(ring);
     uint32_t rslot = 0, rph = 0;                     // ring slot and phase of the next item's first chunk
     unsigned j = 0;
@@ -1171,6 +1175,7 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
     }
   }
   __syncthreads();
+  if (threadIdx.x == 0) finish_counters(a.ctl);
 }
 
 // ---------------------------------------------------------------- host side
@@ -1274,8 +1279,10 @@ size_t counter_bytes(const Plan& plan) {
 cudaError_t launch_apply_simt(const ApplyArgs& a, int nrb, bool adj, int sms, const SimtConfig cfg[2],
                               cudaStream_t stream) {
   sms = std::max(1, sms);
-  cudaError_t err = cudaMemsetAsync(a.counters, 0, counter_bytes(a.plan), stream);
-  if (err != cudaSuccess) return err;
+  if (!a.ctl) {
+    const cudaError_t err = cudaMemsetAsync(a.counters, 0, counter_bytes(a.plan), stream);
+    if (err != cudaSuccess) return err;
+  }
   switch (nrb * 2 + (adj ? 1 : 0)) {
     case 2: return launch_n<1, false>(a, sms, cfg, stream);
     case 3: return launch_n<1, true>(a, sms, cfg, stream);

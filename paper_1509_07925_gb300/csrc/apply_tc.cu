@@ -326,6 +326,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
   const TCPlan& plan = a.plan;
   const int S = plan.n_stages, c = plan.c;
   const uint32_t set_cols = 2u * uint32_t(a.mt_max);   // D1 | D2 of one accumulator set
+  const unsigned n_cnt = unsigned(S) * unsigned(plan.st[0].n_groups);   // (every stage has as many groups)
 
   if (warp == 0 && lane < kAProducers) {
     // ---------------------------------------------------------------- A tiles
@@ -381,10 +382,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     int j = 0;
     RingPos pos;
     bool ok = true;
+    const unsigned* counters = counter_set(a.counters, a.ctl, n_cnt);
     for (int e = 0; e < S && ok; ++e) {
       const TCStage& st = plan.st[e];
       const uint8_t* src = e == 0 ? a.x_in : a.bufs + int64_t(e - 1) * a.buf_stride;
-      const unsigned* cnt_in = a.counters + int64_t(e) * st.n_groups;
+      const unsigned* cnt_in = counters + int64_t(e) * st.n_groups;
       const uint32_t half = uint32_t(st.R8_in) * (TF32 ? 2u * kRow : kRow);
       const uint32_t xhalf = uint32_t(st.K_pad) * kRow;     // hi or lo half of the panel buffer
       const int64_t blk = split_block_bytes(st.R8_in, NR);
@@ -579,6 +581,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     const bool lane_on = NR == 64 || lane < 16;
     const int ri = tl & 1, n = tl >> 1;
     const uint32_t lane_base = uint32_t(32 * quarter) << 16;
+    if (set == 0) clear_other_set(a.counters, a.ctl, n_cnt, unsigned(tid) - 128u, 128u);
     int j = 0;
     bool ok = true;
     for (int e = 0; e < S && ok; ++e) {
@@ -675,13 +678,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     // one fence covers every group stored by then, the two sets' fences overlap, and the
     // epilogue never waits for one.
     const int set = (warp - 12) / 2;
+    unsigned* counters = counter_set(a.counters, a.ctl, n_cnt);
     int j = 0;
     unsigned n = 0, avail = 0;   // groups of this set signalled; seen stored
     bool ok = true;
     for (int e = 0; e + 1 < S && ok; ++e) {
       const TCStage& st = plan.st[e];
       const TCStage& nst = plan.st[e + 1];
-      unsigned* cnt_out = a.counters + int64_t(e + 1) * nst.n_groups;
+      unsigned* cnt_out = counters + int64_t(e + 1) * nst.n_groups;
       for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++j) {
         if (nsets == 2 && (j & 1) != set) continue;
         const SegBlocks out = seg_blocks(st.out_pat, g, st, c);
@@ -721,6 +725,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(taddr));
+  if (tid == 0) finish_counters(a.ctl);
 }
 
 // ------------------------------------------------------------------ leaf kernels
@@ -1160,7 +1165,7 @@ bool leaf_fits(int R8, int c) { return R8 <= kLeafMaxR8 && c <= kLeafMaxC; }
 cudaError_t launch_apply_tc(const TCArgs& a, int grid, size_t smem, cudaStream_t stream, bool tf32, int nr) {
   if (a.nsa < kAProducers || a.nsa % kAProducers != 0) return cudaErrorInvalidValue;
   if (a.nxb < 1 || a.nxb > kMaxXBufs) return cudaErrorInvalidValue;
-  cudaError_t err = cudaSuccess;   // (the caller clears the dependency counters)
+  cudaError_t err = cudaSuccess;
   void (*kern)(TCArgs) = nr == 32 ? (tf32 ? bf_apply_tc<true, 32> : bf_apply_tc<false, 32>)
                                   : (tf32 ? bf_apply_tc<true, 64> : bf_apply_tc<false, 64>);
   if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess)

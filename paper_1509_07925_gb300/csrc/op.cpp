@@ -805,8 +805,6 @@ void apply_tc(mbf_op_s* op, Workspace& w, const float2* g, float2* u, int64_t nr
     // a panel of 32 for the last RHS where they fit one (the host-link input panel keeps 64)
     nr = !host_io && nrhs - r0 <= kTcNRHalf ? kTcNRHalf : kTcNR;
     const bool half = nr == kTcNRHalf;
-    // the tensor kernel's dependency counters (cleared per panel)
-    cuda_check(cudaMemsetAsync(w.tc_counters, 0, tc_counter_bytes(tp), st), "counter clear");
     // page-locked host input: g -> panel in tree order first (rows read across the
     // host link as 16-byte runs); device input: gathered by the leaf kernel itself
     cudaEvent_t e0 = nullptr;
@@ -856,7 +854,8 @@ void apply_tc(mbf_op_s* op, Workspace& w, const float2* g, float2* u, int64_t nr
     ta.bufs = bufs;
     ta.y_out = ylast;
     ta.buf_stride = vec_bytes;
-    ta.counters = w.tc_counters;
+    ta.counters = w.tc_counters + kCtlWords;
+    ta.ctl = w.tc_counters;
     ta.status = w.status;
     ta.nsa = half ? op->tc_nsa32 : op->tc_nsa;
     ta.nxb = half ? op->tc_nxb32 : op->tc_nxb;
@@ -933,8 +932,6 @@ void apply_tc_adj(mbf_op_s* op, Workspace& w, const float2* u, float2* g, int64_
     // a panel of 32 for the last RHS where they fit one (the host-link input panel keeps 64)
     nr = !host_io && nrhs - r0 <= kTcNRHalf ? kTcNRHalf : kTcNR;
     const bool half = nr == kTcNRHalf;
-    // the tensor kernel's dependency counters (cleared per panel)
-    cuda_check(cudaMemsetAsync(w.tc_counters, 0, tc_counter_bytes(ap), st), "counter clear");
     // u -> panel in X-tree order (page-locked host input), or gathered by the leaf kernel
     cudaEvent_t e0 = nullptr;
     if (host_io) {
@@ -979,7 +976,8 @@ void apply_tc_adj(mbf_op_s* op, Workspace& w, const float2* u, float2* g, int64_
     ta.bufs = bufs;
     ta.y_out = ylast;
     ta.buf_stride = vec_bytes;
-    ta.counters = w.tc_counters;
+    ta.counters = w.tc_counters + kCtlWords;
+    ta.ctl = w.tc_counters;
     ta.status = w.status;
     ta.nsa = half ? op->tca_nsa32 : op->tca_nsa;
     ta.nxb = half ? op->tca_nxb32 : op->tca_nxb;
@@ -1052,7 +1050,8 @@ void apply_impl(mbf_op_s* op, const void* in, void* out, int64_t nrhs, int32_t p
   a.in_len = adj ? op->n_out : op->n_in;
   a.out_len = adj ? op->n_in : op->n_out;
   a.bufs = w.bufs;
-  a.counters = w.counters;
+  a.counters = w.counters + kCtlWords;
+  a.ctl = w.counters;
   a.status = w.status;
   a.nrhs = int32_t(nrhs);
   a.xcap = op->xcap;
@@ -1111,21 +1110,34 @@ int64_t tc_vec_bytes(const mbf_op_s* op) {
 void ws_init(const mbf_op_s* op, Workspace& w) {
   const size_t vbytes = size_t(op->plan.n_stages - 1) * size_t(op->positions) * 8 * sizeof(float2);
   if (dev_alloc(&w.bufs, vbytes) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc workspace");
-  if (dev_alloc(&w.counters, counter_bytes(op->plan)) != cudaSuccess || dev_alloc(&w.status, 256) != cudaSuccess)
+  const size_t cnt = counters_alloc(counter_bytes(op->plan));
+  if (dev_alloc(&w.counters, cnt) != cudaSuccess || dev_alloc(&w.status, 256) != cudaSuccess)
     fail(MBF_ERR_OOM, "cudaMalloc counters");
   cuda_check(cudaMemset(w.status, 0, 256), "cudaMemset status");
+  cuda_check(cudaMemset(w.counters, 0, cnt), "cudaMemset counters");
+  cuda_check(cudaStreamSynchronize(nullptr), "cudaMemset counters");   // (the applies' streams may not wait for it)
 }
 
 void ws_prepare_tc(const mbf_op_s* op, Workspace& w) {
-  if (w.tc_bufs || !op->tc_unavailable.empty()) return;
+  if (w.tc_gt || !op->tc_unavailable.empty()) return;   // (the last of the three: all or none)
   const int S = op->tcplan.n_stages;
   const int64_t vec_bytes = tc_vec_bytes(op);
-  if (dev_alloc(&w.tc_bufs, size_t(S + 1) * size_t(vec_bytes)) != cudaSuccess)
-    fail(MBF_ERR_OOM, "cudaMalloc tensor-path workspace");
-  if (dev_alloc(&w.tc_counters, tc_counter_bytes(op->tcplan)) != cudaSuccess)
-    fail(MBF_ERR_OOM, "cudaMalloc tensor-path counters");
-  if (dev_alloc(&w.tc_gt, size_t(std::max<int64_t>({op->n_w, op->n_out, 1})) * kTcNR * sizeof(float2)) != cudaSuccess)
-    fail(MBF_ERR_OOM, "cudaMalloc tensor-path input panel");
+  const size_t cnt = counters_alloc(tc_counter_bytes(op->tcplan));
+  const size_t gt = size_t(std::max<int64_t>({op->n_w, op->n_out, 1})) * kTcNR * sizeof(float2);
+  const char* what = nullptr;
+  if (dev_alloc(&w.tc_bufs, size_t(S + 1) * size_t(vec_bytes)) != cudaSuccess) what = "workspace";
+  else if (dev_alloc(&w.tc_counters, cnt) != cudaSuccess) what = "counters";
+  else if (cudaMemset(w.tc_counters, 0, cnt) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)
+    what = "counters";   // (synchronized: the applies' streams may not wait for the memset)
+  else if (dev_alloc(&w.tc_gt, gt) != cudaSuccess) what = "input panel";
+  if (what) {
+    cudaFree(w.tc_bufs);
+    cudaFree(w.tc_counters);
+    w.tc_bufs = nullptr;
+    w.tc_counters = nullptr;
+    w.tc_gt = nullptr;
+    fail(MBF_ERR_OOM, std::string("cudaMalloc tensor-path ") + what);
+  }
 }
 
 void ws_free(Workspace& w) {

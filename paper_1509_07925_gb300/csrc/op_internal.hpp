@@ -24,7 +24,7 @@ struct RowTable;   // apply.hpp
 // server, so that batches of one operator can run at the same time.
 struct Workspace {
   float2* bufs = nullptr;          // one coefficient vector per stage but the last, 8 RHS wide
-  unsigned* counters = nullptr;    // the dependency counters
+  unsigned* counters = nullptr;    // control words, then two sets of the dependency counters
   int* status = nullptr;
   uint8_t* tc_bufs = nullptr;      // S_main + 1 vectors of c^L blocks x R8 x 64 entries (8 bytes each)
   unsigned* tc_counters = nullptr;
