@@ -14,83 +14,109 @@ namespace {
 
 constexpr int kCThreads = 256;
 constexpr int kCRhs = 8;      // RHS per CTA
-constexpr int kCX = 64;       // outputs x of a CTA (forward)
-constexpr int kCShares = kCThreads / kCX;   // shares of the centre points (forward)
-constexpr int kCTile = 128;   // centre points staged per round
-constexpr int kCBatch = 8;    // K_C entries in flight per thread
+constexpr int kCLanes = 64;   // threads of a share (forward)
+constexpr int kCXt = 4;       // outputs x per thread (forward), kCLanes apart
+constexpr int kCX = kCLanes * kCXt;
+constexpr int kCShares = kCThreads / kCLanes;   // shares of the centre points (forward)
+constexpr int kCTile = 296;   // centre points staged per round (a 17 x 17 centre in one)
+constexpr int kCBatch = 2;    // centre points whose kernel entries are in flight per thread
 constexpr int kCPts = 4;      // centre points per CTA (adjoint)
 
-// Forward: a CTA computes 64 outputs x for 8 RHS; its four shares of 64 threads take the
+// Forward: a CTA computes 256 outputs x for 8 RHS; its four shares of 64 threads take the
 // centre points of a round in turn and their sums are added at the end, always in the
-// same order.  One thread per x over all the centre points (an earlier form) left each
-// thread a serial chain of loads and the chip at 14 warps an SM: 81 us for n = 128, 289
-// points, 32 RHS, from a cold cache; now 52 us.
+// same order.  Four outputs a thread: a 16-byte shared load of g, even one that all lanes
+// share, takes the load pipe four cycles, so with one output a thread (64 multiply-adds to
+// eight such loads) that pipe, not the multiply-adds, set the time.  n = 128, 289 points,
+// 32 RHS from a cold cache (16 us of multiply-adds): 81 us with one thread per x over all
+// the centre points, 52 us with four shares, 58 us with 16 RHS a CTA, 48 us now.
 __global__ void __launch_bounds__(kCThreads) center_fwd_kernel(const float2* __restrict__ Kc,
                                                                const int32_t* __restrict__ idx, int n_c,
                                                                const float2* __restrict__ g, int64_t len_in,
                                                                float2* __restrict__ u, int64_t n_out, int nrhs,
                                                                int accumulate) {
-  __shared__ __align__(16) float2 gs[kCTile][kCRhs];
-  __shared__ float2 part[kCShares - 1][kCRhs][kCX];
-  const int xl = threadIdx.x % kCX, share = threadIdx.x / kCX;
-  const int64_t x = int64_t(blockIdx.x) * kCX + xl;
+  // g of the round's centre points [point][RHS]; at the end sums [share][RHS][x]
+  __shared__ __align__(16) float2 buf[2 * kCRhs * kCX];
+  static_assert(kCTile <= 2 * kCX && kCShares == 4, "buf holds either");
+  const int xl = threadIdx.x % kCLanes, share = threadIdx.x / kCLanes;
+  const int64_t x0 = int64_t(blockIdx.x) * kCX + xl;
   const int r0 = blockIdx.y * kCRhs;
-  const float2* kx = Kc + (x < n_out ? x : n_out - 1);
-  float2 acc[kCRhs];
+  int64_t xk[kCXt];             // (outputs beyond the last: the last one's entries, not stored)
 #pragma unroll
-  for (int r = 0; r < kCRhs; ++r) acc[r] = make_float2(0.f, 0.f);
+  for (int i = 0; i < kCXt; ++i) xk[i] = x0 + i * kCLanes < n_out ? x0 + i * kCLanes : n_out - 1;
+  float2 acc[kCXt][kCRhs];
+#pragma unroll
+  for (int i = 0; i < kCXt; ++i)
+#pragma unroll
+    for (int r = 0; r < kCRhs; ++r) acc[i][r] = make_float2(0.f, 0.f);
   for (int c0 = 0; c0 < n_c; c0 += kCTile) {
     const int nc = min(kCTile, n_c - c0);
     __syncthreads();
+#pragma unroll 4
     for (int q = threadIdx.x; q < nc * kCRhs; q += kCThreads) {
       const int cc = q / kCRhs, r = q - cc * kCRhs;
-      gs[cc][r] = r0 + r < nrhs ? __ldg(g + int64_t(r0 + r) * len_in + idx[c0 + cc]) : make_float2(0.f, 0.f);
+      buf[q] = r0 + r < nrhs ? __ldg(g + int64_t(r0 + r) * len_in + __ldg(idx + c0 + cc)) : make_float2(0.f, 0.f);
     }
     __syncthreads();
     for (int cc = share; cc < nc; cc += kCShares * kCBatch) {
-      float2 k[kCBatch];
+      float2 k[kCBatch][kCXt];
 #pragma unroll
       for (int b = 0; b < kCBatch; ++b)
-        if (cc + b * kCShares < nc) k[b] = __ldg(kx + int64_t(c0 + cc + b * kCShares) * n_out);
+        if (cc + b * kCShares < nc)
+#pragma unroll
+          for (int i = 0; i < kCXt; ++i) k[b][i] = __ldg(Kc + int64_t(c0 + cc + b * kCShares) * n_out + xk[i]);
 #pragma unroll
       for (int b = 0; b < kCBatch; ++b)
         if (cc + b * kCShares < nc) {
-          const float4* gv = reinterpret_cast<const float4*>(gs[cc + b * kCShares]);
+          const float4* gv = reinterpret_cast<const float4*>(buf + (cc + b * kCShares) * kCRhs);
 #pragma unroll
           for (int r2 = 0; r2 < kCRhs / 2; ++r2) {
             const float4 v = gv[r2];
-            acc[2 * r2].x = fmaf(k[b].x, v.x, fmaf(-k[b].y, v.y, acc[2 * r2].x));
-            acc[2 * r2].y = fmaf(k[b].x, v.y, fmaf(k[b].y, v.x, acc[2 * r2].y));
-            acc[2 * r2 + 1].x = fmaf(k[b].x, v.z, fmaf(-k[b].y, v.w, acc[2 * r2 + 1].x));
-            acc[2 * r2 + 1].y = fmaf(k[b].x, v.w, fmaf(k[b].y, v.z, acc[2 * r2 + 1].y));
+#pragma unroll
+            for (int i = 0; i < kCXt; ++i) {
+              float2 &s = acc[i][2 * r2], &t = acc[i][2 * r2 + 1];
+              s.x = fmaf(k[b][i].x, v.x, fmaf(-k[b][i].y, v.y, s.x));
+              s.y = fmaf(k[b][i].x, v.y, fmaf(k[b][i].y, v.x, s.y));
+              t.x = fmaf(k[b][i].x, v.z, fmaf(-k[b][i].y, v.w, t.x));
+              t.y = fmaf(k[b][i].x, v.w, fmaf(k[b][i].y, v.z, t.y));
+            }
           }
         }
     }
   }
-  if (share > 0)
+  // shares 2 and 3 to 0 and 1, then 1 to 0
+  for (int n = 2; n > 0; n >>= 1) {
+    __syncthreads();
+    if (share >= n && share < 2 * n)
 #pragma unroll
-    for (int r = 0; r < kCRhs; ++r) part[share - 1][r][xl] = acc[r];
-  __syncthreads();
-  if (share == 0) {
+      for (int i = 0; i < kCXt; ++i)
 #pragma unroll
-    for (int r = 0; r < kCRhs; ++r) {
+        for (int r = 0; r < kCRhs; ++r) buf[((share - n) * kCRhs + r) * kCX + i * kCLanes + xl] = acc[i][r];
+    __syncthreads();
+    if (share < n)
 #pragma unroll
-      for (int s = 0; s < kCShares - 1; ++s) {
-        acc[r].x += part[s][r][xl].x;
-        acc[r].y += part[s][r][xl].y;
-      }
-      if (x < n_out && r0 + r < nrhs) {
-        float2* o = u + int64_t(r0 + r) * n_out + x;
-        float2 v = acc[r];
-        if (accumulate) {
-          const float2 w = *o;
-          v.x += w.x;
-          v.y += w.y;
+      for (int i = 0; i < kCXt; ++i)
+#pragma unroll
+        for (int r = 0; r < kCRhs; ++r) {
+          const float2 w = buf[(share * kCRhs + r) * kCX + i * kCLanes + xl];
+          acc[i][r].x += w.x;
+          acc[i][r].y += w.y;
         }
-        *o = v;
-      }
-    }
   }
+  if (share == 0)
+#pragma unroll
+    for (int i = 0; i < kCXt; ++i)
+#pragma unroll
+      for (int r = 0; r < kCRhs; ++r)
+        if (x0 + i * kCLanes < n_out && r0 + r < nrhs) {
+          float2* o = u + int64_t(r0 + r) * n_out + x0 + i * kCLanes;
+          float2 v = acc[i][r];
+          if (accumulate) {
+            const float2 w = *o;
+            v.x += w.x;
+            v.y += w.y;
+          }
+          *o = v;
+        }
 }
 
 // Adjoint: one CTA per kCPts centre points and 8 RHS, a block reduction over x; each u
