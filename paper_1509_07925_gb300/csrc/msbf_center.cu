@@ -24,11 +24,10 @@ constexpr int kCPts = 4;      // centre points per CTA (adjoint)
 
 // Forward: a CTA computes 256 outputs x for 8 RHS; its four shares of 64 threads take the
 // centre points of a round in turn and their sums are added at the end, always in the
-// same order.  Four outputs a thread: a 16-byte shared load of g, even one that all lanes
-// share, takes the load pipe four cycles, so with one output a thread (64 multiply-adds to
-// eight such loads) that pipe, not the multiply-adds, set the time.  n = 128, 289 points,
-// 32 RHS from a cold cache (16 us of multiply-adds): 81 us with one thread per x over all
-// the centre points, 52 us with four shares, 58 us with 16 RHS a CTA, 48 us now.
+// same order.  Four outputs a thread, so that a shared load of g serves four of them.
+// n = 128, 289 points, 32 RHS from a cold cache (16 us of multiply-adds): 81 us with one
+// thread per x over all the centre points, 52 us with four shares of one output a thread,
+// 58 us with 16 RHS a CTA, 48 us now.
 __global__ void __launch_bounds__(kCThreads) center_fwd_kernel(const float2* __restrict__ Kc,
                                                                const int32_t* __restrict__ idx, int n_c,
                                                                const float2* __restrict__ g, int64_t len_in,

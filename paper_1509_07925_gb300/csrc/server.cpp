@@ -241,12 +241,12 @@ struct mbf_server_s {
   }
 
   // Factor bytes a group streams: the operator's factors once per pass (a 64-RHS panel
-  // on the tensor cores, up to 4 RHS on the SIMT kernel).  The apply is bound by this
+  // on the tensor cores, up to 8 RHS on the SIMT kernel).  The apply is bound by this
   // traffic, so it sets the group's share of the batch's SMs.
   static double group_work(const mbf_op_s* op, int64_t rhs) {
     if (mbf::uses_tensor(op, rhs, MBF_PREC_AUTO, false))
       return double(std::max<int64_t>(op->tc_bytes, 1)) * double((rhs + 63) / 64);
-    return 8.0 * double(std::max<int64_t>(op->nnz, 1)) * double((rhs + 3) / 4);
+    return 8.0 * double(std::max<int64_t>(op->nnz, 1)) * double((rhs + 7) / 8);
   }
 
   // SMs of each group: the batch's share (grid, or the whole GPU when 0) split by the
