@@ -73,9 +73,10 @@ struct Packer {
 
   int64_t stage_nnz = 0, leaf_x_nnz = 0;   // nonzero entries packed (this stage; U^L items)
 
-  // Append one item: `nlines` lines of `len` entries, value(line, e) -> complex.
+  // Append one item: `nlines` lines of `len` entries, value(line, e) -> complex, in chunks
+  // of max_lpc lines at most.
   template <class F>
-  Item add_item(int nlines, int len, uint8_t kind, uint8_t t, F value) {
+  Item add_item(int nlines, int len, uint8_t kind, uint8_t t, F value, int64_t max_lpc = kMaxChunkLines) {
     Item it{};
     size_t off = (arena.size() + 127) & ~size_t(127);
     if (off / 128 > UINT32_MAX) fail(MBF_ERR_INVALID, "factor arena larger than 512 GB");
@@ -83,7 +84,7 @@ struct Packer {
     it.off128 = uint32_t(off / 128);
     it.nlines = uint16_t(nlines);
     it.len = uint16_t(len);
-    it.lpc = uint16_t(lines_per_chunk(len));
+    it.lpc = uint16_t(std::min<int64_t>(lines_per_chunk(len), std::max<int64_t>(1, max_lpc)));
     it.kind = kind;
     it.t = t;
     const int64_t bytes = item_bytes(nlines, len, it.lpc);
@@ -114,7 +115,16 @@ struct Packer {
   // counts in the item's base, one byte each.
   template <class F>
   Item add_main(const Stage& st, int Rin, int Rout, F value) {
-    if (!st.compact) return add_item(c * Rin, c * Rout, ITEM_MAIN, 0, value);
+    // Where a CTA has a group a stage or less, a stage lasts as long as one block: a multiple
+    // of eight chunks, the same number for each of the SIMT kernel's eight consumer warps.
+    // 2-D DFT n = 64, r = 16, 1 RHS (five chunks of 15 lines): 21.9 us, eight of 8: 21.4, 16 of
+    // 4: 22.6; polar FIO n = 64, r = 24, 5 RHS (ten chunks): 38.7 us, sixteen: 36.9.
+    const auto most = [&](int lines) {
+      if (st.n_groups >= 2 * 152) return int64_t(kMaxChunkLines);
+      const int64_t lpc = lines_per_chunk(c * Rout), n = (lines + lpc - 1) / lpc, n8 = std::max<int64_t>(8, (n + 7) / 8 * 8);
+      return (lines + n8 - 1) / n8;
+    };
+    if (!st.compact) return add_item(c * Rin, c * Rout, ITEM_MAIN, 0, value, most(c * Rin));
     std::vector<int> lines;
     uint32_t counts = 0;
     for (int t = 0; t < c; ++t) {
@@ -129,7 +139,7 @@ struct Packer {
       counts |= uint32_t(r) << (8 * t);
     }
     Item it = add_item(int(lines.size()), c * Rout, ITEM_MAIN, 0,
-                       [&](int line, int e) { return value(lines[size_t(line)], e); });
+                       [&](int line, int e) { return value(lines[size_t(line)], e); }, most(int(lines.size())));
     it.base = int32_t(counts);
     return it;
   }
