@@ -293,7 +293,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
   uint64_t* dempty = dfull + 2;
   uint64_t* done = dempty + 2;
   unsigned* nstored = reinterpret_cast<unsigned*>(done + 1);   // [set][warp]: groups whose outputs the warp has written
-  uint32_t* tslot = nstored + 8;
+  unsigned* nread = nstored + 8;     // groups whose MMAs are done, in order (written by the panel warp)
+  uint32_t* tslot = nread + 1;
   volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
       mbar_init(&dempty[s], 128);
     }
     for (int q = 0; q < 8; ++q) nstored[q] = 0;
+    *nread = 0;
     mbar_init(done, 1);
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -397,6 +399,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
         bool fail = false;
         if (lane == 0) {
           fail = !wait_bar(&xempty[xs], pos.ph ^ 1u, abort);
+          if (!fail && j >= nxb) st_release_cta(nread, unsigned(j - nxb + 1));
           // all c input blocks written by the previous stage
           if (!fail && e > 0) {
             const unsigned* cp = cnt_in + g;
@@ -429,6 +432,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
         }
       }
     }
+    // the last groups' MMAs, for the discard warps
+    if (lane == 0)
+      for (int q = max(j - nxb, 0); q < j && ok; ++q) {
+        ok = wait_bar(&xempty[q % nxb], uint32_t(q / nxb) & 1u, abort);
+        if (ok) st_release_cta(nread, unsigned(q + 1));
+      }
     // wait (bounded) for the copies of the last groups still in flight
     if (lane == 0) {
       for (int q = (j > nxb ? j - nxb : 0); q < j; ++q) {
@@ -439,19 +448,34 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
     }
   } else if (warp == 3 || warp == 13) {
     // ---------------------------------------------------------------- L2 discards
-    // Once a group's MMAs are done (its panel buffer's xempty phase), its c input blocks
+    // Once a group's MMAs are done, its c input blocks
     // are neither in shared memory nor read again: their lines are dropped from L2
     // without a write-back.  Each discard takes a while, so two warps share them.
+    // They follow a count kept by the panel warp, not the buffers' barriers: a discard warp
+    // may fall any number of groups behind, and a barrier's one-bit phase shows one only (a
+    // warp two behind waited for a phase that never came, until its limit of 2 s).
     const int dt = (warp == 3 ? 0 : 32) + lane;
-    RingPos pos;
+    unsigned n = 0, avail = 0;
     bool ok = true;
     for (int e = 0; e < S && ok; ++e) {
       const TCStage& st = plan.st[e];
       const uint8_t* src = e == 0 ? a.x_in : a.bufs + int64_t(e - 1) * a.buf_stride;
       const int64_t blk = split_block_bytes(st.R8_in, NR);
-      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, pos.next(nxb)) {
+      for (int g = blockIdx.x; g < st.n_groups && ok; g += gridDim.x, ++n) {
         const SegBlocks in = seg_blocks(st.in_pat, g, st, c);
-        if (!__all_sync(0xffffffffu, wait_bar(&xempty[pos.i], pos.ph, abort))) {
+        uint64_t t0 = 0;
+        for (unsigned k = 1; avail <= n && (avail = ld_acquire_cta(nread)) <= n; ++k) {
+          __nanosleep(100);
+          if ((k & 63u) == 0) {
+            const uint64_t t = gtimer();
+            if (t0 == 0) t0 = t;
+            if (*abort || t - t0 > kTimeoutNs) {
+              ok = false;
+              break;
+            }
+          }
+        }
+        if (!__all_sync(0xffffffffu, ok)) {
           ok = false;
           break;
         }

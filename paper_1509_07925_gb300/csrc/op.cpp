@@ -1077,7 +1077,7 @@ void apply_impl(mbf_op_s* op, const void* in, void* out, int64_t nrhs, int32_t p
     cuda_check(cudaMemsetAsync(out, 0, size_t(nrhs) * size_t(op->n_in) * sizeof(float2), st), "cudaMemsetAsync");
   const int sms = grid > 0 ? std::min(grid, op->sms) : op->sms;
   for (int64_t r0 = 0; r0 < nrhs;) {
-    const int nrb = simt_pass_rhs(nrhs - r0);
+    const int nrb = std::min(simt_pass_rhs(nrhs - r0), w.simt_rhs);
     a.rhs0 = int32_t(r0);
     a.buf_stride = op->positions * nrb;
     cudaEvent_t e0 = prof_begin(op, st);
@@ -1118,8 +1118,14 @@ int64_t tc_vec_bytes(const mbf_op_s* op) {
 // (or through tc_prepare / the server before a capture), so later applies allocate
 // nothing.
 void ws_init(const mbf_op_s* op, Workspace& w) {
-  const size_t vbytes = size_t(op->plan.n_stages - 1) * size_t(op->positions) * 8 * sizeof(float2);
-  if (dev_alloc(&w.bufs, vbytes) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc workspace");
+  // vectors for passes of 8 RHS, or of 4 where the device has no room for those
+  const size_t vbytes = size_t(op->plan.n_stages - 1) * size_t(op->positions) * sizeof(float2);
+  w.simt_rhs = 8;
+  if (dev_alloc(&w.bufs, vbytes * 8) != cudaSuccess) {
+    cudaGetLastError();
+    w.simt_rhs = 4;
+    if (dev_alloc(&w.bufs, vbytes * 4) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc workspace");
+  }
   const size_t cnt = counters_alloc(counter_bytes(op->plan));
   if (dev_alloc(&w.counters, cnt) != cudaSuccess || dev_alloc(&w.status, 256) != cudaSuccess)
     fail(MBF_ERR_OOM, "cudaMalloc counters");

@@ -23,7 +23,8 @@ struct RowTable;   // apply.hpp
 // use).  An operator owns one, and lends further ones from a pool it keeps to the
 // server, so that batches of one operator can run at the same time.
 struct Workspace {
-  float2* bufs = nullptr;          // one coefficient vector per stage but the last, 8 RHS wide
+  float2* bufs = nullptr;          // one coefficient vector per stage but the last, simt_rhs wide
+  int simt_rhs = 8;                // most RHS of a SIMT pass (8, or 4 where memory is short)
   unsigned* counters = nullptr;    // control words, then two sets of the dependency counters
   int* status = nullptr;
   uint8_t* tc_bufs = nullptr;      // S_main + 1 vectors of c^L blocks x R8 x 64 entries (8 bytes each)

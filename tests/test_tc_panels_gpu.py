@@ -69,3 +69,31 @@ def test_multiscale_sum_with_narrow_panels(bd, nrhs):
         u = ut.cpu().numpy()
         assert max(rel(u[k], ref[k]) for k in range(nrhs)) <= TOL_BF16X3, (nrhs, adjoint)
     gm.close()
+
+
+def test_small_sm_share_ends_without_a_wait_running_out(bd):
+    """1024 groups per level on the few SMs of a served batch's share: over a hundred groups
+    a CTA and level, so that every role of the kernel may run many groups ahead of another;
+    no request takes anywhere near the 2 s after which a device wait gives up."""
+    import time
+    hf = bd.HostFactors.build(2, 64, 6, 8)
+    op = bd.Operator(hf)
+    g = torch.from_numpy(complex_normal(64 * 64, 64, seed=61).astype(np.complex64)).cuda()
+    ref = torch.empty_like(g)
+    st = torch.cuda.current_stream().cuda_stream
+    op.apply(g.data_ptr(), ref.data_ptr(), 64, MBF_PREC_BF16X3, st)
+    op.check(st)
+    srv = bd.Server(staging_budget_bytes=1 << 28, max_inflight=16, max_batch_rhs=64)
+    outs = [torch.zeros_like(g) for _ in range(48)]
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    for k, u in enumerate(outs):
+        srv.submit(op, g.data_ptr(), u.data_ptr(), 64 if k % 2 else 20)
+    srv.drain(30.0)
+    elapsed = time.perf_counter() - t0
+    srv.close()
+    assert elapsed < 1.0, elapsed
+    for k, u in enumerate(outs):
+        n = 64 if k % 2 else 20
+        assert torch.linalg.norm(u[:n] - ref[:n]) <= 2e-4 * torch.linalg.norm(ref[:n])
+    op.close()
