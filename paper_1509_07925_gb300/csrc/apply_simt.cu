@@ -23,11 +23,11 @@
 // group's chain hides the other's.  A group to a warp, as before, had 1/8 of the SM's
 // bandwidth and a private ring of three slots for it: every stage ended in a wait for
 // streams.  Polar FIO n = 256, L = 6, r = 24 (389 MB of factors), one RHS: 110.6 us with a
-// group to a warp, 111 us with a group to a CTA of 8 warps and one CTA to an SM, 82 us
-// with two CTAs of 4 (4.7 TB/s); adjoint 280 -> 111 us (16-byte loads, 16 totals reduced
-// over the lanes in 16 exchanges instead of 5 each); n = 128 with 7 RHS 472 -> 155 us (one
-// pass of 8 instead of 4 + 3); n = 64, L = 4 with 5 RHS 199 -> 41 us; 2-D DFT n = 64, L = 4,
-// r = 16, one RHS 50 -> 22 us.
+// group to a warp, 111 us with a group to a CTA of 8 warps and one CTA to an SM, 80 us
+// with two CTAs of 4 (4.85 TB/s); adjoint 280 -> 115 us (16-byte loads, 16 totals reduced
+// over the lanes in 16 exchanges instead of 5 each); n = 128 with 7 RHS 473 -> 148 us (one
+// pass of 8 instead of 4 + 3); n = 64, L = 4 with 5 RHS 203 -> 37 us; 2-D DFT n = 64, L = 4,
+// r = 16, one RHS 51 -> 21 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>

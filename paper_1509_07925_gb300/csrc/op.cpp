@@ -51,6 +51,18 @@ cudaError_t dev_alloc(T** p, size_t bytes) {
   return cudaMalloc(p, bytes);
 }
 
+// Zero device memory now, on a stream of its own: the applies' streams may not wait for the
+// default stream, and one of them may be capturing.
+cudaError_t zero_now(void* p, size_t bytes) {
+  cudaStream_t st = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(p, 0, bytes, st);
+  const cudaError_t e2 = cudaStreamSynchronize(st);
+  cudaStreamDestroy(st);
+  return e != cudaSuccess ? e : e2;
+}
+
 template <class T>
 T* dev_upload(const std::vector<T>& v, const char* what) {
   T* p = nullptr;
@@ -1130,8 +1142,7 @@ void ws_init(const mbf_op_s* op, Workspace& w) {
   if (dev_alloc(&w.counters, cnt) != cudaSuccess || dev_alloc(&w.status, 256) != cudaSuccess)
     fail(MBF_ERR_OOM, "cudaMalloc counters");
   cuda_check(cudaMemset(w.status, 0, 256), "cudaMemset status");
-  cuda_check(cudaMemset(w.counters, 0, cnt), "cudaMemset counters");
-  cuda_check(cudaStreamSynchronize(nullptr), "cudaMemset counters");   // (the applies' streams may not wait for it)
+  cuda_check(zero_now(w.counters, cnt), "clearing the counters");
 }
 
 void ws_prepare_tc(const mbf_op_s* op, Workspace& w) {
@@ -1143,8 +1154,7 @@ void ws_prepare_tc(const mbf_op_s* op, Workspace& w) {
   const char* what = nullptr;
   if (dev_alloc(&w.tc_bufs, size_t(S + 1) * size_t(vec_bytes)) != cudaSuccess) what = "workspace";
   else if (dev_alloc(&w.tc_counters, cnt) != cudaSuccess) what = "counters";
-  else if (cudaMemset(w.tc_counters, 0, cnt) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)
-    what = "counters";   // (synchronized: the applies' streams may not wait for the memset)
+  else if (zero_now(w.tc_counters, cnt) != cudaSuccess) what = "counters";
   else if (dev_alloc(&w.tc_gt, gt) != cudaSuccess) what = "input panel";
   if (what) {
     cudaFree(w.tc_bufs);
