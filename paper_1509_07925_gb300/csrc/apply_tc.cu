@@ -116,6 +116,10 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
+// Orders this thread's view of global memory between the generic proxy (loads, stores,
+// atomics) and the async proxy (bulk copies): a block stored by another CTA's epilogue and
+// read here by a bulk copy needs one on the way, beside the release and the acquire.
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 // Shared-memory matrix descriptor: start, leading (K-direction core-matrix) and
 // stride (M/N-direction) byte offsets, fixed bit 46, no swizzle.
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
@@ -420,10 +424,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
           if (fail) *abort = 1;
           else mbar_expect_tx(&xfull[xs], uint32_t(kParts * c) * half);
         }
-        if (__shfl_sync(0xffffffffu, fail ? 1 : 0, 0)) {   // (also orders the expect before the copies)
+        if (__shfl_sync(0xffffffffu, fail ? 1 : 0, 0)) {
           ok = false;
           break;
         }
+        // lane 0's acquire holds for the copying lanes (a shuffle orders no memory), and their
+        // copies, in the async proxy, come after the generic stores that it acquired
+        __syncwarp();
+        fence_proxy_async_global();
         if (lane < kParts * c) {
           const int t = lane / kParts, hl = lane - t * kParts;
           const uint8_t* sb = src + int64_t(in.base + t * in.step) * blk;
@@ -738,6 +746,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) bf_apply_tc(const __grid_consta
           avail = __reduce_min_sync(0xffffffffu, avail);   // what all four warps have stored
           __syncwarp();
           __threadfence();
+          fence_proxy_async_global();                      // (the consumers read by bulk copies)
         }
         if (lane < c) atomicAdd(cnt_out + consumer, 1u);
         ++n;
