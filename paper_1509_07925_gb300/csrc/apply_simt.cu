@@ -23,11 +23,15 @@
 // group's chain hides the other's.  A group to a warp, as before, had 1/8 of the SM's
 // bandwidth and a private ring of three slots for it: every stage ended in a wait for
 // streams.  Polar FIO n = 256, L = 6, r = 24 (389 MB of factors), one RHS: 110.6 us with a
-// group to a warp, 111 us with a group to a CTA of 8 warps and one CTA to an SM, 80 us
-// with two CTAs of 4 (4.85 TB/s); adjoint 280 -> 115 us (16-byte loads, 16 totals reduced
-// over the lanes in 16 exchanges instead of 5 each); n = 128 with 7 RHS 473 -> 148 us (one
-// pass of 8 instead of 4 + 3); n = 64, L = 4 with 5 RHS 203 -> 37 us; 2-D DFT n = 64, L = 4,
-// r = 16, one RHS 51 -> 21 us.
+// group to a warp, 111 us with a group to a CTA of 8 warps and one CTA to an SM, 76 us
+// with two CTAs of 4 (5.08 TB/s); adjoint 280 -> 117 us (16-byte loads, 16 totals reduced
+// over the lanes in 16 exchanges instead of 5 each); n = 128 with 7 RHS 472 -> 144 us (one
+// pass of 8 instead of 4 + 3); n = 64, L = 4 with 5 RHS 199 -> 36 us; 2-D DFT n = 64, L = 4,
+// r = 16, one RHS 50 -> 20 us.  Many small blocks, where a group to a warp did best: 2-D DFT
+// n = 64, L = 6 with 1 and 2 RHS, r = 4 44.5 / 46.5 -> 43.6 / 46.2 us, r = 8 46.7 / 50.6 ->
+// 43.7 / 48.7; n = 256, L = 8, r = 4 654 / 776 -> 655 / 757 (the many lines side by side of such
+// blocks are added in pairs; one after another they took r = 4 to 55.1 / 61.2 and 876 / 1002).
+// The kernels of 4 and 8 RHS spill 40 to 160 bytes (128 registers a thread).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -93,22 +97,16 @@ __device__ __forceinline__ void set_status(int* status, volatile int* abort, int
   *abort = 1;
 }
 
-__device__ __forceinline__ int64_t pat_off(int pat, int g, int t, const Stage& s, int R, int c) {
-  const int a = g / s.B, b = g - (g / s.B) * s.B;
-  if (pat == PAT_SPLIT) return (int64_t(c * a + t) * s.B + b) * R;
-  if (pat == PAT_CONTIG) return (int64_t(c) * g + t) * R;
-  return (int64_t(c * b + t) * s.ch + a) * R;  // PAT_CORNER
-}
+// B, c^h and c are powers of two: the group and segment maps are shifts (a division each for
+// the gather and signal warps cost 4 us of 48 over the 7 stages of n = 64, L = 6).
+__device__ __forceinline__ int lg2(int x) { return 31 - __clz(x); }
 
 // The group of stage `s` whose input pattern `pat` reads segment P (position P * R).
-__device__ __forceinline__ int pat_group(int pat, int64_t P, const Stage& s, int c) {
-  if (pat == PAT_CONTIG) return int(P / c);
-  if (pat == PAT_SPLIT) {
-    const int64_t q = P / s.B;
-    return int((q / c) * s.B + (P - q * s.B));
-  }
-  const int64_t q = P / s.ch;   // PAT_CORNER: P = (c b + t) ch + a, g = a B + b
-  return int((P - q * s.ch) * s.B + q / c);
+__device__ __forceinline__ int pat_group(int pat, int P, const Stage& s, int c) {
+  const int lc = lg2(c), lb = lg2(s.B);
+  if (pat == PAT_CONTIG) return P >> lc;
+  if (pat == PAT_SPLIT) return (((P >> lb) >> lc) << lb) + (P & (s.B - 1));
+  return ((P & (s.ch - 1)) << lb) + ((P >> lg2(s.ch)) >> lc);   // PAT_CORNER: P = (c b + t) ch + a, g = a B + b
 }
 
 __device__ __forceinline__ bool item_ok(const Item& it) {
@@ -175,7 +173,7 @@ struct SegMap {
 };
 __device__ __forceinline__ SegMap seg_map(int pat, int g, const Stage& s, int R, int c) {
   if (pat == PAT_CONTIG) return {c * g * R, R};
-  const int a = g / s.B, b = g - a * s.B;
+  const int a = g >> lg2(s.B), b = g & (s.B - 1);
   if (pat == PAT_SPLIT) return {(c * a * s.B + b) * R, s.B * R};
   return {(c * b * s.ch + a) * R, s.ch * R};         // PAT_CORNER
 }
@@ -416,6 +414,7 @@ __host__ __device__ constexpr int entry_parts(int len) { return len > 128 ? 2 : 
 template <int NRB, bool ADJ, int W, int GA, int CPS>
 __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __grid_constant__ ApplyArgs a) {
   static_assert(W == 4 || W == 8, "consumer warps");
+  static_assert(GA % 2 == 0, "the partial sums start 16-byte aligned for any xcap");
   constexpr int LW = W == 8 ? 3 : 2;
   constexpr int NR = NRB;
   const uint64_t dep_lim = a.wait_ns ? a.wait_ns : kTimeoutNs;
@@ -511,7 +510,7 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
         const int ci = c0 + lane;
         bool pend = lane < n;
         uint64_t t0 = 0;
-        for (unsigned tries = 1; __any_sync(0xffffffffu, pend); ++tries) {
+        for (unsigned tries = 1;; ++tries) {
           if (pend && mbar_test(&empty[slot], ph)) {
             const uint32_t bytes = ci == nch - 1 ? tb : cb;
             mbar_expect_tx(&full[slot], bytes);
@@ -519,6 +518,7 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
             latest[slot] = (ph ^ 1u) + 1u;
             pend = false;
           }
+          if (!__any_sync(0xffffffffu, pend)) break;
           __nanosleep(40);                           // (leaves the shared-memory pipe to the products)
           if ((tries & 63u) == 0) {
             bool stop = *abort != 0;
@@ -582,8 +582,8 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
           __threadfence();
         }
         if (lane < c) {
-          const int64_t P = pat_off(out_pat, g, lane, st, 1, c);
-          atomicAdd(cnt_out + pat_group(next_in, P, nst, c), 1u);
+          const SegMap sm = seg_map(out_pat, g, st, 1, c);
+          atomicAdd(cnt_out + pat_group(next_in, sm.base + lane * sm.step, nst, c), 1u);
         }
       }
     }
@@ -606,13 +606,13 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
       const unsigned* cnt_in = counters + int64_t(e) * st.n_groups;
       for (int g = first_group(e); g < st.n_groups && ok; g += grid, ++j) {
         if (int(j % GA) != gw) continue;
+        Item myit{};                                 // (in flight while the buffer is waited for)
+        if (lane < st.n_items)
+          myit = a.items[st.item_base + int64_t(g) * st.n_items + (ADJ ? st.n_items - 1 - lane : lane)];
         if (!__all_sync(0xffffffffu, wait_bar(&xempty[gw], ((j / GA) & 1u) ^ 1u, a, abort, lim, ST_EMPTY_TIMEOUT))) {
           ok = false;
           break;
         }
-        Item myit{};
-        if (lane < st.n_items)
-          myit = a.items[st.item_base + int64_t(g) * st.n_items + (ADJ ? st.n_items - 1 - lane : lane)];
         if (__any_sync(0xffffffffu, lane < st.n_items && !item_ok(myit))) {
           if (lane == 0) set_status(a.status, abort, ST_BAD_ITEM);
           ok = false;
@@ -697,7 +697,11 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
           V* dv = reinterpret_cast<V*>(xin);
           const V* from[U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) from[u] = sv + int64_t(place(min(lane + 32 * u, max(nq, 1) - 1) / H)) * H + lane % H;
+          for (int u = 0; u < U; ++u)
+            // (one RHS forward: not for batches that a small block does not fill; elsewhere the test
+            // costs more than it saves, 8 RHS n = 128: 144 us without it, 156 with)
+            if (ADJ || NRB > 1 || u == 0 || 32 * u < nq)
+              from[u] = sv + int64_t(place(min(lane + 32 * u, max(nq, 1) - 1) / H)) * H + lane % H;
           // wait until the group's c input segments have been counted in
           bool got = true;
           const unsigned* cp = cnt_in + g;
@@ -942,20 +946,23 @@ __global__ void __launch_bounds__((W + GA + 2) * 32, CPS) bf_apply_simt(const __
               }
             });
             if constexpr (kVec) {
-              // add the side-by-side lines, then the warp's sums go to its share of `red`: float4
-              // units [share][pair of values][column], a column a lane
-              for (int t = 1; t < LPW; ++t)
+              // add the side-by-side lines in pairs, then pairs of pairs ... (up to 32 lines of rows of
+              // four entries), then the warp's sums go to its share of `red`: float4 units
+              // [share][pair of values][column], a column a lane
+              for (int t = 1; t < LPW; t *= 2) {
+                const bool add = (s_line & (2 * t - 1)) == 0 && s_line + t < LPW;
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
                   for (int r = 0; r < NR; ++r) {
                     const float px = __shfl_sync(0xffffffffu, acc[i][r].x, (lane + t * G) & 31);
                     const float py = __shfl_sync(0xffffffffu, acc[i][r].y, (lane + t * G) & 31);
-                    if (s_line == 0) {
+                    if (add) {
                       acc[i][r].x += px;
                       acc[i][r].y += py;
                     }
                   }
+              }
               float4* red4 = reinterpret_cast<float4*>(red);
               if (s_line == 0 && lane_on)
 #pragma unroll
