@@ -51,18 +51,6 @@ cudaError_t dev_alloc(T** p, size_t bytes) {
   return cudaMalloc(p, bytes);
 }
 
-// Zero device memory now, on a stream of its own: the applies' streams may not wait for the
-// default stream, and one of them may be capturing.
-cudaError_t zero_now(void* p, size_t bytes) {
-  cudaStream_t st = nullptr;
-  cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(p, 0, bytes, st);
-  const cudaError_t e2 = cudaStreamSynchronize(st);
-  cudaStreamDestroy(st);
-  return e != cudaSuccess ? e : e2;
-}
-
 template <class T>
 T* dev_upload(const std::vector<T>& v, const char* what) {
   T* p = nullptr;
@@ -754,6 +742,8 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
     }
     if (!op->simt_unavailable.empty() && !op->tc_unavailable.empty())
       fail(MBF_ERR_INVALID, "no apply path: SIMT (" + op->simt_unavailable + "), tensor cores (" + op->tc_unavailable + ")");
+    // the uploads came from pageable memory, so the last of them may still be under way
+    cuda_check(cudaStreamSynchronize(nullptr), "uploads");
   } catch (...) {
     op_free(op);
     throw;
@@ -1101,6 +1091,16 @@ void apply_impl(mbf_op_s* op, const void* in, void* out, int64_t nrhs, int32_t p
 
 }  // namespace
 
+cudaError_t zero_now(void* p, size_t bytes) {
+  cudaStream_t st = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(p, 0, bytes, st);
+  const cudaError_t e2 = cudaStreamSynchronize(st);
+  cudaStreamDestroy(st);
+  return e != cudaSuccess ? e : e2;
+}
+
 void validate(const mbf_factors_t& f) { validate_factors(f); }
 
 void set_last_error(const std::string& m) { g_last_error = m; }
@@ -1141,7 +1141,7 @@ void ws_init(const mbf_op_s* op, Workspace& w) {
   const size_t cnt = counters_alloc(counter_bytes(op->plan));
   if (dev_alloc(&w.counters, cnt) != cudaSuccess || dev_alloc(&w.status, 256) != cudaSuccess)
     fail(MBF_ERR_OOM, "cudaMalloc counters");
-  cuda_check(cudaMemset(w.status, 0, 256), "cudaMemset status");
+  cuda_check(zero_now(w.status, 256), "clearing the status word");
   cuda_check(zero_now(w.counters, cnt), "clearing the counters");
 }
 
@@ -1583,7 +1583,7 @@ mbf_status mbf_op_check(mbf_op_t op, void* stream) {
     int st = 0;
     cuda_check(cudaMemcpy(&st, op->ws.status, sizeof(int), cudaMemcpyDeviceToHost), "read status");
     if (st != ST_OK) {
-      cuda_check(cudaMemset(op->ws.status, 0, sizeof(int)), "clear status");
+      cuda_check(zero_now(op->ws.status, sizeof(int)), "clear status");
       static const char* names[] = {"ok", "grid barrier", "full mbarrier", "empty mbarrier", "bad item",
                                     "dependency counter"};
       fail(MBF_ERR_TIMEOUT, std::string("device wait gave up: ") + (st >= 0 && st <= 5 ? names[st] : "unknown"));

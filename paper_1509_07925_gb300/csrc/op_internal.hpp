@@ -117,6 +117,10 @@ struct mbf_op_s {
 
 namespace mbf {
 void set_last_error(const std::string& m);
+// Zero device memory now, on a stream of its own: a clear on the default stream may return
+// before it has run, the applies' streams may not wait for it, and one of them may be
+// capturing.
+cudaError_t zero_now(void* p, size_t bytes);
 // Internal entry points shared with the server and the tuner.  All throw mbf::Error.
 bool uses_tensor(const mbf_op_s* op, int64_t nrhs, int32_t precision, bool adj);
 void tc_prepare(mbf_op_s* op);

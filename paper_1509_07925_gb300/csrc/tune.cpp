@@ -131,7 +131,7 @@ extern "C" mbf_status mbf_op_tune(mbf_op_t op, void* stream, mbf_tune_result_t* 
     int dev_status = 0;
     cuda_ok(cudaMemcpy(&dev_status, op->ws.status, sizeof(int), cudaMemcpyDeviceToHost), "status");
     if (dev_status != 0) {
-      cudaMemset(op->ws.status, 0, sizeof(int));
+      cuda_ok(mbf::zero_now(op->ws.status, sizeof(int)), "clear status");
       fail(MBF_ERR_TIMEOUT, "a device wait gave up while tuning");
     }
   });
