@@ -21,10 +21,13 @@ struct Error : std::runtime_error {
 };
 [[noreturn]] inline void fail(mbf_status c, const std::string& m) { throw Error(c, m); }
 void set_last_error(const std::string& m);
+void clear_cuda_error();
 
 // Runs fn at the C ABI boundary: an mbf::Error becomes its status, a failed host
 // allocation MBF_ERR_OOM and any other exception MBF_ERR_INVALID; mbf_last_error() then
 // returns the message ("" after a success).  No exception crosses the ABI.
+// A CUDA error that is reported so is not left behind as the runtime's last error, where the
+// next check of a launch, here or in the caller's own code, would find it.
 template <class F>
 mbf_status abi_guard(F&& fn) noexcept {
   try {
@@ -32,6 +35,7 @@ mbf_status abi_guard(F&& fn) noexcept {
     set_last_error("");
     return MBF_OK;
   } catch (const Error& e) {
+    if (e.code == MBF_ERR_CUDA || e.code == MBF_ERR_OOM) clear_cuda_error();
     set_last_error(e.what());
     return e.code;
   } catch (const std::bad_alloc&) {

@@ -48,7 +48,9 @@ cudaError_t dev_alloc(T** p, size_t bytes) {
       break;
     }
   }
-  return cudaMalloc(p, bytes);
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();   // (the callers report it, or do without)
+  return e;
 }
 
 template <class T>
@@ -1104,6 +1106,7 @@ cudaError_t zero_now(void* p, size_t bytes) {
 void validate(const mbf_factors_t& f) { validate_factors(f); }
 
 void set_last_error(const std::string& m) { g_last_error = m; }
+void clear_cuda_error() { cudaGetLastError(); }
 
 // Which path an apply takes: split-BF16x3 or TF32 on request; AUTO uses the split-BF16x3
 // tensor cores from tc_min_rhs right-hand sides (8, or what the tuner measured), for the
@@ -1134,7 +1137,6 @@ void ws_init(const mbf_op_s* op, Workspace& w) {
   const size_t vbytes = size_t(op->plan.n_stages - 1) * size_t(op->positions) * sizeof(float2);
   w.simt_rhs = 8;
   if (dev_alloc(&w.bufs, vbytes * 8) != cudaSuccess) {
-    cudaGetLastError();
     w.simt_rhs = 4;
     if (dev_alloc(&w.bufs, vbytes * 4) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc workspace");
   }
