@@ -1478,6 +1478,7 @@ mbf_status mbf_apply_host(mbf_op_t op, const void* g_host, void* u_host, int64_t
       cuda_check(cudaStreamSynchronize(st), "sync");
       cudaFree(op->d_stage_in);
       op->d_stage_in = nullptr;
+      op->stage_in_bytes = 0;
       if (dev_alloc(&op->d_stage_in, in_b) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc staging");
       op->stage_in_bytes = in_b;
     }
@@ -1485,6 +1486,7 @@ mbf_status mbf_apply_host(mbf_op_t op, const void* g_host, void* u_host, int64_t
       cuda_check(cudaStreamSynchronize(st), "sync");
       cudaFree(op->d_stage_out);
       op->d_stage_out = nullptr;
+      op->stage_out_bytes = 0;
       if (dev_alloc(&op->d_stage_out, out_b) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc staging");
       op->stage_out_bytes = out_b;
     }

@@ -45,3 +45,12 @@ def test_a_refused_allocation_leaves_no_error_behind(bd_op):
     op.apply(g.data_ptr(), out[1].data_ptr(), 64, bd.MBF_PREC_BF16X3, st)
     op.check(st)
     assert torch.equal(torch.view_as_real(out[0]), torch.view_as_real(out[1]))
+
+
+def test_staging_is_allocated_again_after_a_refusal(bd_op):
+    """The refused larger staging buffer took the place of the one there was."""
+    bd, op = bd_op
+    g = complex_normal(N * N, 2, seed=82).astype(np.complex64)
+    ref = op.apply_host(g, 2, bd.MBF_PREC_FP32_SIMT)
+    _refused(bd, op)
+    assert np.array_equal(op.apply_host(g, 2, bd.MBF_PREC_FP32_SIMT), ref)
