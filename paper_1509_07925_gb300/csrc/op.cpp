@@ -744,6 +744,7 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
     }
     if (!op->simt_unavailable.empty() && !op->tc_unavailable.empty())
       fail(MBF_ERR_INVALID, "no apply path: SIMT (" + op->simt_unavailable + "), tensor cores (" + op->tc_unavailable + ")");
+    ws_widen(op, op->ws);
     // the uploads came from pageable memory, so the last of them may still be under way
     cuda_check(cudaStreamSynchronize(nullptr), "uploads");
   } catch (...) {
@@ -1129,22 +1130,32 @@ int64_t tc_vec_bytes(const mbf_op_s* op) {
   return Tree::ipow(op->c, op->L) * split_block_bytes(r8max);
 }
 
+// Bytes of the SIMT path's vectors for one RHS.
+static size_t simt_vec_bytes(const mbf_op_s* op) {
+  return size_t(op->plan.n_stages - 1) * size_t(op->positions) * sizeof(float2);
+}
+
 // Workspaces.  The SIMT parts at operator creation; the tensor path's on its first use
 // (or through tc_prepare / the server before a capture), so later applies allocate
 // nothing.
 void ws_init(const mbf_op_s* op, Workspace& w) {
-  // vectors for passes of 8 RHS, or of 4 where the device has no room for those
-  const size_t vbytes = size_t(op->plan.n_stages - 1) * size_t(op->positions) * sizeof(float2);
-  w.simt_rhs = 8;
-  if (dev_alloc(&w.bufs, vbytes * 8) != cudaSuccess) {
-    w.simt_rhs = 4;
-    if (dev_alloc(&w.bufs, vbytes * 4) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc workspace");
-  }
+  w.simt_rhs = 4;
+  if (dev_alloc(&w.bufs, simt_vec_bytes(op) * 4) != cudaSuccess) fail(MBF_ERR_OOM, "cudaMalloc workspace");
   const size_t cnt = counters_alloc(counter_bytes(op->plan));
   if (dev_alloc(&w.counters, cnt) != cudaSuccess || dev_alloc(&w.status, 256) != cudaSuccess)
     fail(MBF_ERR_OOM, "cudaMalloc counters");
   cuda_check(zero_now(w.status, 256), "clearing the status word");
   cuda_check(zero_now(w.counters, cnt), "clearing the counters");
+}
+
+// Vectors for passes of 8 RHS in the place of those for 4, where the device has room for them
+// beside everything else that the operator needs: asked for last, and done without.
+void ws_widen(const mbf_op_s* op, Workspace& w) {
+  float2* wide = nullptr;
+  if (dev_alloc(&wide, simt_vec_bytes(op) * 8) != cudaSuccess) return;
+  cudaFree(w.bufs);
+  w.bufs = wide;
+  w.simt_rhs = 8;
 }
 
 void ws_prepare_tc(const mbf_op_s* op, Workspace& w) {
@@ -1229,6 +1240,8 @@ Workspace* ws_acquire(mbf_op_s* op, bool tensor) {
       auto* nw = new Workspace();
       try {
         ws_init(op, *nw);
+        if (tensor) ws_prepare_tc(op, *nw);
+        ws_widen(op, *nw);
       } catch (...) {
         ws_free(*nw);
         delete nw;

@@ -24,7 +24,7 @@ struct RowTable;   // apply.hpp
 // server, so that batches of one operator can run at the same time.
 struct Workspace {
   float2* bufs = nullptr;          // one coefficient vector per stage but the last, simt_rhs wide
-  int simt_rhs = 8;                // most RHS of a SIMT pass (8, or 4 where memory is short)
+  int simt_rhs = 4;                // most RHS of a SIMT pass (8, or 4 where memory is short)
   unsigned* counters = nullptr;    // control words, then two sets of the dependency counters
   int* status = nullptr;
   uint8_t* tc_bufs = nullptr;      // S_main + 1 vectors of c^L blocks x R8 x 64 entries (8 bytes each)
@@ -124,9 +124,11 @@ cudaError_t zero_now(void* p, size_t bytes);
 // Internal entry points shared with the server and the tuner.  All throw mbf::Error.
 bool uses_tensor(const mbf_op_s* op, int64_t nrhs, int32_t precision, bool adj);
 void tc_prepare(mbf_op_s* op);
-// Allocate a workspace for `op` (its SIMT parts; ws_prepare_tc adds the tensor path's,
-// once) and free one.  Throw mbf::Error (MBF_ERR_OOM) on a failed allocation.
+// Allocate a workspace for `op` (its SIMT parts for passes of 4 RHS; ws_prepare_tc adds the
+// tensor path's, once, and ws_widen room for passes of 8, if there is any) and free one.
+// Throw mbf::Error (MBF_ERR_OOM) on a failed allocation, ws_widen does not.
 void ws_init(const mbf_op_s* op, Workspace& w);
+void ws_widen(const mbf_op_s* op, Workspace& w);
 void ws_prepare_tc(const mbf_op_s* op, Workspace& w);
 void ws_free(Workspace& w);
 // Borrow a workspace of `op` for one apply in flight (its own one if free, else one of its
