@@ -387,12 +387,14 @@ mbf_status mbf_msbf_destroy(mbf_msbf_t m);
 /* ------------------------------------------------------------------ autotuner
  * The paper has no counterpart (its applies are single-threaded CPU loops).  Measures,
  * on `stream` with device buffers it allocates and frees itself, (a) the FP32 SIMT apply
- * for 1, 2, 4, 8, 16, 32 and 64 RHS, (b) the tensor-core apply of one 64-RHS panel for
- * two or three panel buffers, each with the even A-tile ring depths 2 .. 16 that fit
- * shared memory beside them (8 configurations at most), then keeps the fastest and
- * sets the RHS count from which MBF_PREC_AUTO takes the tensor cores to the smallest
- * measured count at which one panel is faster than the SIMT apply.  Blocking; the
- * operator must be idle.  The choices stay with the operator until it is destroyed. */
+ * for 1, 2, 4, 8, 16, 32 and 64 RHS, (b) the tensor-core apply of one panel of 64 RHS and
+ * of one of 32 (which 32 and fewer RHS take) in the present configuration and for two or
+ * three panel buffers, each with the deepest even A-tile ring depths, 16 at most, that fit
+ * shared memory beside them (8 configurations at most), then keeps each panel's fastest,
+ * the present one where none is faster, and sets the RHS count from which MBF_PREC_AUTO
+ * takes the tensor cores to the smallest measured count at which its panel is faster than
+ * the SIMT apply.  Blocking; the operator must be idle.  The choices stay with the operator
+ * until it is destroyed. */
 typedef struct mbf_tune_result {
   int32_t n_simt;
   int32_t simt_rhs[8];
@@ -403,11 +405,20 @@ typedef struct mbf_tune_result {
                                    panel_buffers[i] panel buffers                    */
   int32_t tc_slots_chosen;      /* 0 if the tensor path is unavailable               */
   int32_t tc_min_rhs;           /* AUTO uses the tensor cores from this many RHS     */
-  int32_t panel_buffers[8];     /* panel buffers of configuration i (2 or 3)          */
+  int32_t panel_buffers[8];     /* panel buffers of configuration i (1 to 3)          */
   int32_t tc_buffers_chosen;    /* panel buffers kept                                 */
   int32_t reserved_tune;
 } mbf_tune_result_t;
 mbf_status mbf_op_tune(mbf_op_t op, void* stream, mbf_tune_result_t* out);
+/* The tuner's rules as pure host functions (for tests; no device).  Candidates: for a panel
+ * that has `slots` ring slots and `buffers` panel buffers now, and deepest[b - 1] slots at
+ * most beside b buffers (0: none), the n (8 at most) configurations it times, the present
+ * one first.  Crossover: from the SIMT times of n RHS counts in increasing order and those
+ * of a panel of 32 and of 64 RHS, the RHS count it sets (65: none). */
+mbf_status mbf_debug_tune_candidates(int32_t slots, int32_t buffers, const int32_t* deepest, int32_t* n,
+                                     int32_t* slots_out, int32_t* buffers_out);
+mbf_status mbf_debug_tune_crossover(int32_t n, const int32_t* rhs, const double* simt_ms, double narrow_ms,
+                                    double full_ms, int32_t* min_rhs);
 
 /* ------------------------------------------------------------------ serving
  * The paper has no counterpart.  A server owns a worker thread, a few CUDA streams

@@ -147,6 +147,10 @@ SIGNATURES = {
     "mbf_apply_static": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p]),
     "mbf_op_set_profiling": (C.c_int, [C.c_void_p, C.c_int32]),
     "mbf_op_tune": (C.c_int, [C.c_void_p, C.c_void_p, C.POINTER(TuneResult)]),
+    "mbf_debug_tune_candidates": (C.c_int, [C.c_int32, C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
+                                            C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
+    "mbf_debug_tune_crossover": (C.c_int, [C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_double), C.c_double,
+                                           C.c_double, C.POINTER(C.c_int32)]),
     "mbf_build_msbf": (C.c_int, [C.POINTER(Problem), C.c_void_p, C.c_void_p, C.POINTER(BuildOpts), C.c_int32,
                                  C.POINTER(C.c_void_p)]),
     "mbf_msbf_create": (C.c_int, [C.POINTER(C.c_void_p), C.c_int32, C.c_void_p, C.c_void_p, C.c_int64,
@@ -518,6 +522,24 @@ def split_sms(work, share):
     out = (C.c_int32 * max(1, n))()
     _check(lib().mbf_debug_split_sms(a_w, n, share, out))
     return list(out)[:n]
+
+
+def tune_candidates(slots, buffers, deepest):
+    """(ring slots, panel buffers) that the autotuner times for a panel configured as
+    (slots, buffers), with deepest[b - 1] slots at most beside b buffers
+    (mbf_debug_tune_candidates)."""
+    d, n, s, b = (C.c_int32 * 3)(*deepest), C.c_int32(), (C.c_int32 * 8)(), (C.c_int32 * 8)()
+    _check(lib().mbf_debug_tune_candidates(slots, buffers, d, C.byref(n), s, b))
+    return list(zip(s, b))[:n.value]
+
+
+def tune_crossover(rhs, simt_ms, narrow_ms, full_ms):
+    """RHS count from which the autotuner lets AUTO take the tensor cores
+    (mbf_debug_tune_crossover)."""
+    n, out = len(rhs), C.c_int32()
+    _check(lib().mbf_debug_tune_crossover(n, (C.c_int32 * max(1, n))(*rhs), (C.c_double * max(1, n))(*simt_ms),
+                                          narrow_ms, full_ms, C.byref(out)))
+    return out.value
 
 
 class Server:
