@@ -224,7 +224,8 @@ typedef struct mbf_op_info {
   int64_t bytes_algorithmic;    /* 8 * nnz_algorithmic (complex64)                        */
   int64_t bytes_packed;         /* device bytes of the packed tiles incl. padding         */
   int64_t bytes_stage[32];      /* packed bytes streamed by each forward stage            */
-  int32_t grid, threads, smem;  /* persistent launch shape of the SIMT apply              */
+  int32_t grid, threads, smem;  /* launch shape of a SIMT apply of one RHS on the whole GPU:
+                                   CTAs, threads and shared memory of one                 */
   int64_t nnz_stage[32];        /* nonzero factor entries applied by each forward stage    */
   int64_t nnz_leaf_u;           /* of which U^L (part of the last stage)                  */
   int32_t tensor_ok;            /* 1 if the tensor-core path is available                 */

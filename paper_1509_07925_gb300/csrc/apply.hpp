@@ -155,7 +155,13 @@ struct LeafArgs {
 };
 
 // FP32 SIMT path (apply_simt.cu): one launch per pass of 1, 2, 4 or 8 RHS.
-int simt_threads();
+// The launch of a pass over plans of `groups` groups on `sms` SMs: one CTA to an SM or two.
+struct SimtShape {
+  bool pair;
+  int grid, threads;
+  size_t smem;
+};
+SimtShape simt_shape(int groups, int sms, const SimtConfig cfg[2]);
 int simt_pass_rhs(int64_t rhs_left);   // RHS of the next pass (the last one may be padded)
 cudaError_t simt_config(int nrb, int xcap, SimtConfig cfg[2]);
 cudaError_t launch_apply_simt(const ApplyArgs& a, int nrb, bool adj, int sms, const SimtConfig cfg[2],

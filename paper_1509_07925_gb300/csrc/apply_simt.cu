@@ -1241,18 +1241,21 @@ constexpr int kWideWarps = 8, kWideGathers = 4, kPairWarps = 4, kPairGathers = 2
 
 template <int NRB, bool ADJ>
 cudaError_t launch_n(const ApplyArgs& a, int sms, const SimtConfig cfg[2], cudaStream_t stream) {
-  const int groups = a.plan.st[0].n_groups;   // (the same for every stage)
-  // Two CTAs to an SM where each gets at least a group per stage: a group's chain of
-  // waits, gathers and reductions on one overlaps the other's products.  Fewer groups
-  // than that are finished soonest by the most warps.
-  if (cfg[1].slots > 0 && groups >= 2 * sms)
-    return launch_t<NRB, ADJ, kPairWarps, kPairGathers, 2>(a, 2 * sms, cfg[1], stream);
-  return launch_t<NRB, ADJ, kWideWarps, kWideGathers, 1>(a, std::min(sms, groups), cfg[0], stream);
+  const SimtShape s = simt_shape(a.plan.st[0].n_groups, sms, cfg);   // (as many groups in every stage)
+  if (s.pair) return launch_t<NRB, ADJ, kPairWarps, kPairGathers, 2>(a, s.grid, cfg[1], stream);
+  return launch_t<NRB, ADJ, kWideWarps, kWideGathers, 1>(a, s.grid, cfg[0], stream);
 }
 
 }  // namespace
 
-int simt_threads() { return (kWideWarps + kWideGathers + 2) * 32; }
+// Two CTAs to an SM where each gets at least a group per stage: a group's chain of waits,
+// gathers and reductions on one overlaps the other's products.  Fewer groups than that are
+// finished soonest by the most warps.
+SimtShape simt_shape(int groups, int sms, const SimtConfig cfg[2]) {
+  if (cfg[1].slots > 0 && groups >= 2 * sms)
+    return {true, 2 * sms, (kPairWarps + kPairGathers + 2) * 32, cfg[1].smem};
+  return {false, std::min(sms, groups), (kWideWarps + kWideGathers + 2) * 32, cfg[0].smem};
+}
 
 int simt_pass_rhs(int64_t rhs_left) { return rhs_left > 4 ? 8 : rhs_left > 2 ? 4 : rhs_left == 2 ? 2 : 1; }
 

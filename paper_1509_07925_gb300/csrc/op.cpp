@@ -1412,9 +1412,10 @@ mbf_status mbf_op_info(mbf_op_t op, mbf_op_info_t* info) {
     info->bytes_algorithmic = 8 * op->nnz;
     info->bytes_packed = op->bytes_packed;
     for (int s = 0; s < op->plan.n_stages && s < 32; ++s) info->bytes_stage[s] = op->plan.st[s].bytes;
-    info->grid = op->sms;
-    info->threads = simt_threads();
-    info->smem = int(op->simt[1][0].smem);
+    const SimtShape shape = simt_shape(op->plan.st[0].n_groups, op->sms, op->simt[1]);
+    info->grid = shape.grid;
+    info->threads = shape.threads;
+    info->smem = int(shape.smem);
     for (size_t e = 0; e < op->nnz_stage.size() && e < 32; ++e) info->nnz_stage[e] = op->nnz_stage[e];
     info->nnz_leaf_u = op->nnz_leaf_x;
     info->tensor_ok = op->tc_unavailable.empty() ? 1 : 0;
