@@ -18,7 +18,7 @@ constexpr int kCLanes = 64;   // threads of a share (forward)
 constexpr int kCXt = 4;       // outputs x per thread (forward), kCLanes apart
 constexpr int kCX = kCLanes * kCXt;
 constexpr int kCShares = kCThreads / kCLanes;   // shares of the centre points (forward)
-constexpr int kCTile = 296;   // centre points staged per round (a 17 x 17 centre in one)
+constexpr int kCTile = 512;   // centre points staged per round (what the buffer holds)
 constexpr int kCBatch = 2;    // centre points whose kernel entries are in flight per thread
 constexpr int kCPts = 4;      // centre points per CTA (adjoint)
 
