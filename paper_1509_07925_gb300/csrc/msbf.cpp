@@ -17,7 +17,7 @@
 #include "op_internal.hpp"
 
 struct mbf_msbf_s {
-  int device = 0;
+  int device = 0, sms = 0;
   std::vector<mbf_op_s*> parts;
   std::vector<int32_t> part_t, part_L;
   bool own = false;
@@ -41,6 +41,11 @@ void msbf_free(mbf_msbf_s* m) {
   cudaFree(m->d_Kc);
   cudaFree(m->d_idx);
   delete m;
+}
+
+void device_of(mbf_msbf_s* m) {
+  cuda_ok(cudaGetDevice(&m->device), "cudaGetDevice");
+  cuda_ok(cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, m->device), "attr");
 }
 
 // Upload the centre: Kc host complex128 [n_c][n_out] (c-major), idx [n_c].
@@ -93,7 +98,7 @@ mbf_status mbf_msbf_create(const mbf_op_t* parts, int32_t n_parts, const double*
     if (n_parts == 0 && n_center_points == 0) fail(MBF_ERR_INVALID, "empty multiscale operator");
     auto* m = new mbf_msbf_s();
     try {
-      cuda_ok(cudaGetDevice(&m->device), "cudaGetDevice");
+      device_of(m);
       for (int32_t i = 0; i < n_parts; ++i) {
         if (!parts[i]) fail(MBF_ERR_INVALID, "NULL part");
         if (i == 0) {
@@ -135,7 +140,7 @@ mbf_status mbf_build_msbf(const mbf_problem_t* prob, mbf_entry_fn fn, void* ctx,
     auto* m = new mbf_msbf_s();
     m->own = true;
     try {
-      cuda_ok(cudaGetDevice(&m->device), "cudaGetDevice");
+      device_of(m);
       m->n_out = m->n_in = N;
       std::vector<int64_t> centre;
       for (int64_t p = 0; p < N; ++p)
@@ -201,7 +206,7 @@ mbf_status mbf_msbf_apply(mbf_msbf_t m, const void* g, void* u, int64_t nrhs, in
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // centre first (it initialises u), then every corona's BF adds into u
     cuda_ok(mbf::launch_center_fwd(m->d_Kc, m->d_idx, int(m->n_c), static_cast<const float2*>(g), m->n_in,
-                                   static_cast<float2*>(u), m->n_out, int(nrhs), false, st),
+                                   static_cast<float2*>(u), m->n_out, int(nrhs), false, m->sms, st),
             "centre launch");
     for (mbf_op_s* p : m->parts) mbf::apply_dev(p, g, u, nrhs, precision, st, false, 0, true);
   });

@@ -22,12 +22,11 @@ constexpr int kCTile = 512;   // centre points staged per round (what the buffer
 constexpr int kCBatch = 2;    // centre points whose kernel entries are in flight per thread
 constexpr int kCPts = 4;      // centre points per CTA (adjoint)
 
-// Forward: a CTA computes 256 outputs x for 8 RHS; its four shares of 64 threads take the
-// centre points of a round in turn and their sums are added at the end, always in the
-// same order.  Four outputs a thread, so that a shared load of g serves four of them.
-// n = 128, 289 points, 32 RHS from a cold cache (16 us of multiply-adds): 81 us with one
-// thread per x over all the centre points, 52 us with four shares of one output a thread,
-// 58 us with 16 RHS a CTA, 48 us now.
+// Forward, few CTAs: a CTA computes 256 outputs x for 8 RHS; its four shares of 64 threads
+// take the centre points of a round in turn and their sums are added at the end, always in
+// the same order.  Four outputs a thread, so that a shared load of g serves four of them.
+// n = 128, 289 points, 32 RHS from a cold cache (16 us of multiply-adds): 88 us with one
+// thread per x over all the centre points, 53 us so (58 us with 16 RHS a CTA).
 __global__ void __launch_bounds__(kCThreads) center_fwd_kernel(const float2* __restrict__ Kc,
                                                                const int32_t* __restrict__ idx, int n_c,
                                                                const float2* __restrict__ g, int64_t len_in,
@@ -118,6 +117,54 @@ __global__ void __launch_bounds__(kCThreads) center_fwd_kernel(const float2* __r
         }
 }
 
+// Forward, many CTAs: one output a thread over all the centre points, so that six CTAs share
+// an SM (42 registers; two of the kernel above) and hide one another's loads.
+__global__ void __launch_bounds__(kCThreads) center_fwd_many_kernel(const float2* __restrict__ Kc,
+                                                                    const int32_t* __restrict__ idx, int n_c,
+                                                                    const float2* __restrict__ g, int64_t len_in,
+                                                                    float2* __restrict__ u, int64_t n_out, int nrhs,
+                                                                    int accumulate) {
+  __shared__ float2 gs[kCTile][kCRhs];
+  const int64_t x = int64_t(blockIdx.x) * kCX + threadIdx.x;
+  const int r0 = blockIdx.y * kCRhs;
+  static_assert(kCX == kCThreads, "one output a thread");
+  float2 acc[kCRhs];
+#pragma unroll
+  for (int r = 0; r < kCRhs; ++r) acc[r] = make_float2(0.f, 0.f);
+  for (int c0 = 0; c0 < n_c; c0 += kCTile) {
+    const int nc = min(kCTile, n_c - c0);
+    __syncthreads();
+    for (int q = threadIdx.x; q < nc * kCRhs; q += kCThreads) {
+      const int cc = q / kCRhs, r = q - cc * kCRhs;
+      gs[cc][r] = r0 + r < nrhs ? __ldg(g + int64_t(r0 + r) * len_in + idx[c0 + cc]) : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    if (x < n_out)
+      for (int cc = 0; cc < nc; ++cc) {
+        const float2 k = __ldg(Kc + int64_t(c0 + cc) * n_out + x);
+#pragma unroll
+        for (int r = 0; r < kCRhs; ++r) {
+          const float2 v = gs[cc][r];
+          acc[r].x = fmaf(k.x, v.x, fmaf(-k.y, v.y, acc[r].x));
+          acc[r].y = fmaf(k.x, v.y, fmaf(k.y, v.x, acc[r].y));
+        }
+      }
+  }
+  if (x >= n_out) return;
+#pragma unroll
+  for (int r = 0; r < kCRhs; ++r) {
+    if (r0 + r >= nrhs) break;
+    float2* o = u + int64_t(r0 + r) * n_out + x;
+    float2 v = acc[r];
+    if (accumulate) {
+      const float2 w = *o;
+      v.x += w.x;
+      v.y += w.y;
+    }
+    *o = v;
+  }
+}
+
 // Adjoint: one CTA per kCPts centre points and 8 RHS, a block reduction over x; each u
 // value read serves all the CTA's centre points.
 __global__ void __launch_bounds__(kCThreads) center_adj_kernel(const float2* __restrict__ Kc,
@@ -175,13 +222,18 @@ __global__ void __launch_bounds__(kCThreads) center_adj_kernel(const float2* __r
 }  // namespace
 
 cudaError_t launch_center_fwd(const float2* Kc, const int32_t* idx, int n_c, const float2* g, int64_t len_in,
-                              float2* u, int64_t n_out, int nrhs, bool accumulate, cudaStream_t st) {
+                              float2* u, int64_t n_out, int nrhs, bool accumulate, int sms, cudaStream_t st) {
   if (n_c == 0) {
     if (accumulate) return cudaSuccess;
     return cudaMemsetAsync(u, 0, size_t(nrhs) * size_t(n_out) * sizeof(float2), st);
   }
   const dim3 grid(unsigned((n_out + kCX - 1) / kCX), unsigned((nrhs + kCRhs - 1) / kCRhs));
-  center_fwd_kernel<<<grid, kCThreads, 0, st>>>(Kc, idx, n_c, g, len_in, u, n_out, nrhs, accumulate ? 1 : 0);
+  // four shares a CTA up to the two CTAs to an SM that they leave room for; beyond those one
+  // output a thread.  us of either with 256, 512 and 2048 CTAs: n = 128, 81 points 22 / 30,
+  // 37 / 31; 289 points 53 / 88, 94 / 92; n = 256, 289 points 63 / 107, 113 / 109, 361 / 301.
+  // (Between 768 and 1024 CTAs the shares are at times faster, 553 / 678 us at 1089 points.)
+  const auto kern = int64_t(grid.x) * grid.y <= 2 * int64_t(sms) ? center_fwd_kernel : center_fwd_many_kernel;
+  kern<<<grid, kCThreads, 0, st>>>(Kc, idx, n_c, g, len_in, u, n_out, nrhs, accumulate ? 1 : 0);
   return cudaGetLastError();
 }
 
