@@ -223,7 +223,7 @@ mbf_status mbf_msbf_apply_adjoint(mbf_msbf_t m, const void* u, void* g, int64_t 
     // the parts and the centre write disjoint entries of g (they partition Omega)
     cuda_ok(cudaMemsetAsync(g, 0, size_t(nrhs) * size_t(m->n_in) * sizeof(float2), st), "cudaMemsetAsync");
     cuda_ok(mbf::launch_center_adj(m->d_Kc, m->d_idx, int(m->n_c), static_cast<const float2*>(u), m->n_out,
-                                   static_cast<float2*>(g), m->n_in, int(nrhs), st),
+                                   static_cast<float2*>(g), m->n_in, int(nrhs), m->sms, st),
             "centre launch");
     for (mbf_op_s* p : m->parts) mbf::apply_dev(p, u, g, nrhs, precision, st, true, 0, true);
   });

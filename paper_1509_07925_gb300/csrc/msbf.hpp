@@ -12,6 +12,6 @@ cudaError_t launch_center_fwd(const float2* Kc, const int32_t* idx, int n_c, con
                               float2* u, int64_t n_out, int nrhs, bool accumulate, int sms, cudaStream_t st);
 // g[r][idx[c]] += sum_x conj(Kc[c][x]) u[r][x].
 cudaError_t launch_center_adj(const float2* Kc, const int32_t* idx, int n_c, const float2* u, int64_t n_out,
-                              float2* g, int64_t len_in, int nrhs, cudaStream_t st);
+                              float2* g, int64_t len_in, int nrhs, int sms, cudaStream_t st);
 
 }  // namespace mbf

@@ -20,7 +20,6 @@ constexpr int kCX = kCLanes * kCXt;
 constexpr int kCShares = kCThreads / kCLanes;   // shares of the centre points (forward)
 constexpr int kCTile = 512;   // centre points staged per round (what the buffer holds)
 constexpr int kCBatch = 2;    // centre points whose kernel entries are in flight per thread
-constexpr int kCPts = 4;      // centre points per CTA (adjoint)
 
 // Forward, few CTAs: a CTA computes 256 outputs x for 8 RHS; its four shares of 64 threads
 // take the centre points of a round in turn and their sums are added at the end, always in
@@ -165,28 +164,29 @@ __global__ void __launch_bounds__(kCThreads) center_fwd_many_kernel(const float2
   }
 }
 
-// Adjoint: one CTA per kCPts centre points and 8 RHS, a block reduction over x; each u
+// Adjoint: one CTA per P centre points and 8 RHS, a block reduction over x; each u
 // value read serves all the CTA's centre points.
+template <int P>
 __global__ void __launch_bounds__(kCThreads) center_adj_kernel(const float2* __restrict__ Kc,
                                                                const int32_t* __restrict__ idx, int n_c,
                                                                const float2* __restrict__ u, int64_t n_out,
                                                                float2* __restrict__ g, int64_t len_in, int nrhs) {
-  __shared__ float2 red[kCThreads / 32][kCPts][kCRhs];
-  const int c0 = blockIdx.x * kCPts, r0 = blockIdx.y * kCRhs;
-  float2 acc[kCPts][kCRhs];
+  __shared__ float2 red[kCThreads / 32][P][kCRhs];
+  const int c0 = blockIdx.x * P, r0 = blockIdx.y * kCRhs;
+  float2 acc[P][kCRhs];
 #pragma unroll
-  for (int p = 0; p < kCPts; ++p)
+  for (int p = 0; p < P; ++p)
 #pragma unroll
     for (int r = 0; r < kCRhs; ++r) acc[p][r] = make_float2(0.f, 0.f);
   for (int64_t x = threadIdx.x; x < n_out; x += kCThreads) {
-    float2 k[kCPts], v[kCRhs];
+    float2 k[P], v[kCRhs];
 #pragma unroll
-    for (int p = 0; p < kCPts; ++p) k[p] = __ldg(Kc + int64_t(min(c0 + p, n_c - 1)) * n_out + x);   // use conj(k)
+    for (int p = 0; p < P; ++p) k[p] = __ldg(Kc + int64_t(min(c0 + p, n_c - 1)) * n_out + x);   // use conj(k)
 #pragma unroll
     for (int r = 0; r < kCRhs; ++r)
       v[r] = r0 + r < nrhs ? __ldg(u + int64_t(r0 + r) * n_out + x) : make_float2(0.f, 0.f);
 #pragma unroll
-    for (int p = 0; p < kCPts; ++p)
+    for (int p = 0; p < P; ++p)
 #pragma unroll
       for (int r = 0; r < kCRhs; ++r) {
         acc[p][r].x = fmaf(k[p].x, v[r].x, fmaf(k[p].y, v[r].y, acc[p][r].x));
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kCThreads) center_adj_kernel(const float2* __r
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int p = 0; p < kCPts; ++p)
+  for (int p = 0; p < P; ++p)
 #pragma unroll
     for (int r = 0; r < kCRhs; ++r) {
       float sx = acc[p][r].x, sy = acc[p][r].y;
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kCThreads) center_adj_kernel(const float2* __r
     }
   __syncthreads();
   const int p = int(threadIdx.x) / kCRhs, r = int(threadIdx.x) % kCRhs;
-  if (p < kCPts && c0 + p < n_c && r0 + r < nrhs) {
+  if (p < P && c0 + p < n_c && r0 + r < nrhs) {
     float2 s = make_float2(0.f, 0.f);
     for (int w = 0; w < kCThreads / 32; ++w) {
       s.x += red[w][p][r].x;
@@ -238,10 +238,17 @@ cudaError_t launch_center_fwd(const float2* Kc, const int32_t* idx, int n_c, con
 }
 
 cudaError_t launch_center_adj(const float2* Kc, const int32_t* idx, int n_c, const float2* u, int64_t n_out,
-                              float2* g, int64_t len_in, int nrhs, cudaStream_t st) {
+                              float2* g, int64_t len_in, int nrhs, int sms, cudaStream_t st) {
   if (n_c == 0) return cudaSuccess;
-  const dim3 grid(unsigned((n_c + kCPts - 1) / kCPts), unsigned((nrhs + kCRhs - 1) / kCRhs));
-  center_adj_kernel<<<grid, kCThreads, 0, st>>>(Kc, idx, n_c, u, n_out, g, len_in, nrhs);
+  // four centre points a CTA, or two where that leaves fewer CTAs than SMs.  us with two and
+  // with four: n = 128, 289 points, 8 RHS (73 CTAs of four) 53 and 57, 32 RHS (292) 108 and 59;
+  // n = 64, 1 RHS 18 and 20; n = 256, 1089 points (273) 386 and 245 us.  (One point a CTA,
+  // the RHS loop cut at nrhs: 117, 196, 18 and 418 us.)
+  const int y = (nrhs + kCRhs - 1) / kCRhs;
+  const bool few = int64_t((n_c + 3) / 4) * y < sms;
+  const dim3 grid(unsigned(few ? (n_c + 1) / 2 : (n_c + 3) / 4), unsigned(y));
+  const auto kern = few ? center_adj_kernel<2> : center_adj_kernel<4>;
+  kern<<<grid, kCThreads, 0, st>>>(Kc, idx, n_c, u, n_out, g, len_in, nrhs);
   return cudaGetLastError();
 }
 
