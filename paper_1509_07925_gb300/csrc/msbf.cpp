@@ -63,6 +63,7 @@ void upload_centre(mbf_msbf_s* m, const double* Kc, const int64_t* idx, int64_t 
   cuda_ok(cudaMemcpy(m->d_Kc, k.data(), k.size() * sizeof(float2), cudaMemcpyHostToDevice), "upload centre kernel");
   cuda_ok(cudaMalloc(&m->d_idx, ix.size() * sizeof(int32_t)), "cudaMalloc centre index");
   cuda_ok(cudaMemcpy(m->d_idx, ix.data(), ix.size() * sizeof(int32_t), cudaMemcpyHostToDevice), "upload centre index");
+  cuda_ok(cudaStreamSynchronize(nullptr), "uploads");   // (from pageable memory: it may still be under way)
 }
 
 // Corona index of each Omega point (eq. domaindecomp): n/2^(t+2) < max_k |xi_k| <= n/2^(t+1),
