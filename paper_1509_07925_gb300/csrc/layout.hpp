@@ -31,6 +31,9 @@ constexpr int kMaxStages = 24;
 constexpr int kMaxLen = 256;           // longest line (c R) the consumers handle
 constexpr int kMaxLeaf = 1024;         // most points in one leaf
 constexpr int kMaxChunkLines = 256;   // lines per chunk (bounds the per-chunk leaf gather)
+// Groups from which the packer takes the SIMT kernel to run two CTAs to an SM (simt_shape
+// decides by the device's SMs; a GB300 has 152; packed data does not depend on the device).
+constexpr int kPackPairGroups = 2 * 152;
 constexpr uint64_t kTimeoutNs = 2000000000ull;   // 2 s limit on every device-side wait
 
 enum Pattern : int32_t {

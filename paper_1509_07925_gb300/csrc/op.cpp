@@ -117,12 +117,14 @@ struct Packer {
   // counts in the item's base, one byte each.
   template <class F>
   Item add_main(const Stage& st, int Rin, int Rout, F value) {
-    // Where a CTA has a group a stage or less, a stage lasts as long as one block: a multiple
-    // of eight chunks, the same number for each of the SIMT kernel's eight consumer warps.
-    // 2-D DFT n = 64, r = 16, 1 RHS (five chunks of 15 lines): 21.9 us, eight of 8: 21.4, 16 of
-    // 4: 22.6; polar FIO n = 64, r = 24, 5 RHS (ten chunks): 38.7 us, sixteen: 36.9.
+    // Where a CTA has a group a stage or less, a stage lasts as long as one block: about a
+    // multiple of eight chunks (as near as equal line counts come: 20 lines give seven, 100
+    // fifteen), for the SIMT kernel's eight consumer warps.  2-D DFT n = 64, r = 16, 1 RHS
+    // (five chunks of 15 lines): 21.9 us, eight of 8: 21.4, 16 of 4: 22.6; polar FIO n = 64,
+    // r = 24, 5 RHS (ten chunks): 38.7 us, sixteen: 36.9; n = 32, L = 4, r = 8, the adjoint with
+    // 5 RHS: 43.5 and 28.5.
     const auto most = [&](int lines) {
-      if (st.n_groups >= 2 * 152) return int64_t(kMaxChunkLines);
+      if (st.n_groups >= kPackPairGroups) return int64_t(kMaxChunkLines);
       const int64_t lpc = lines_per_chunk(c * Rout), n = (lines + lpc - 1) / lpc, n8 = std::max<int64_t>(8, (n + 7) / 8 * 8);
       return (lines + n8 - 1) / n8;
     };
@@ -623,6 +625,7 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
     check_plan(op->plan, pk.items, pk.arena.size(), op->positions, f, &op->simt_unavailable);
     // ---- device side
     cuda_check(cudaGetDevice(&op->device), "cudaGetDevice");
+    cuda_check(cudaDeviceGetAttribute(&op->sms, cudaDevAttrMultiProcessorCount, op->device), "attr");
     op->d_arena = dev_upload(pk.arena, "factor arena");
     op->d_items = dev_upload(pk.items, "item table");
     auto to32 = [](const int64_t* p, int64_t n) {
@@ -639,7 +642,7 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
     // for a tree whose largest group holds more than twice the mean of the non-empty ones,
     // and where the groups alone would leave SMs idle (64 groups of 256 points, 32 RHS:
     // 47 us a CTA per group)
-    const bool few = nL / op->c < 2 * 152;
+    const bool few = nL / op->c < 2 * op->sms;
     auto ragged = [&](const int64_t* off) {
       int64_t mx = 0, tot = 0, ne = 0;
       for (int64_t gq = 0; gq < nL / op->c; ++gq) {
@@ -681,7 +684,6 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
         op->xcap = std::max<int>(op->xcap, int(std::min<int64_t>(off[(gq + 1) * op->c] - off[gq * op->c], kMaxGroupPoints)));
     for (int nrb : {1, 2, 4, 8})
       cuda_check(simt_config(nrb, op->xcap, op->simt[nrb]), "simt_config");
-    cuda_check(cudaDeviceGetAttribute(&op->sms, cudaDevAttrMultiProcessorCount, op->device), "attr");
     // tensor-core tiles (the multi-RHS path); an operator whose tiles do not fit keeps
     // the SIMT path only and says why
     try {
