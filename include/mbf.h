@@ -294,15 +294,15 @@ mbf_status mbf_apply_host_batch(mbf_op_t op, const void* g_host, void* u_host, i
  * to a fixed budget, or latency-critical loops where an allocation (which may
  * synchronize the device) is not allowed.  Same arguments and result as
  * mbf_apply with precision MBF_PREC_FP32_SIMT; the coefficient workspace and the
- * grid-barrier counter live in one fixed 4 MiB device array that the library
- * reserves on every device that loads it, until the process exits.
- *   - Needs 256 + 4 * (stages * c^(L-1)) (rounded up to 256) + stages * 8 * (c^L * max
+ * dependency counters live in one fixed 4 MiB device array that the library reserves
+ * on every device that loads it, until the process exits.
+ *   - Needs 256 (padding) + 4 * (stages * c^(L-1)) (rounded up to 256) + stages * 8 * (c^L * max
  *     rank) * (RHS per pass: 1, 2 or 4) bytes, stages = 2 (L - L/2) + 1; more returns
  *     MBF_ERR_INVALID and launches nothing.
  *   - The first call on each device looks up the array's device address on that
  *     device (cudaGetSymbolAddress); make that first call before any stream capture.
- *   - All calls share the array, which keeps the last call's contents; the barrier
- *     counter is cleared at the start of every call.  Calls that overlap on the GPU
+ *   - All calls share the array, which keeps the last call's contents; the counters are
+ *     cleared at the start of every pass.  Calls that overlap on the GPU
  *     race on the array: serialize them.  Device waits that run out of time are
  *     reported by mbf_op_check on `op`, as for mbf_apply. */
 mbf_status mbf_apply_static(mbf_op_t op, const void* g, void* u, int64_t nrhs, void* stream);
@@ -313,8 +313,8 @@ mbf_status mbf_op_check(mbf_op_t op, void* stream);
  * stage >= 0, later FP32 SIMT applies on this operator make the dependency wait of
  * group 0 of that stage (execution order, 1 .. n_stages - 1) wait for one producer more
  * than the plan has, so that the wait can only end by running out of time; wait_ns > 0
- * shortens every wait of those applies on a dependency counter, the pass barrier or a
- * chunk copy from 2 s to wait_ns.  The apply then stops early, its output undefined,
+ * shortens every wait of those applies on a dependency counter from 2 s to wait_ns, and
+ * those inside a CTA from 4 s to twice wait_ns.  The apply then stops early, its output undefined,
  * and mbf_op_check reports MBF_ERR_TIMEOUT, as for a real stall.  stage = -1 and
  * wait_ns = 0 restore normal applies.  MBF_ERR_INVALID for a stage beyond the plan or a
  * negative limit. */

@@ -86,11 +86,10 @@ __device__ __forceinline__ void finish_counters(unsigned* ctl) {
 
 enum DeviceStatus : int {
   ST_OK = 0,
-  ST_BARRIER_TIMEOUT = 1,
-  ST_FULL_TIMEOUT = 2,
-  ST_EMPTY_TIMEOUT = 3,
-  ST_BAD_ITEM = 4,
-  ST_DEP_TIMEOUT = 5
+  ST_FULL_TIMEOUT = 1,
+  ST_EMPTY_TIMEOUT = 2,
+  ST_BAD_ITEM = 3,
+  ST_DEP_TIMEOUT = 4
 };
 
 

@@ -10,7 +10,7 @@
 // resident operator using only memory the library reserved when it was loaded.
 //
 // Limits and sharing: the array holds kStaticScratchBytes (4 MiB) on every device
-// that loads the library, for the life of the process.  A call needs 256 bytes, one
+// that loads the library, for the life of the process.  A call needs 256 bytes of padding, one
 // dependency counter per group of every stage, and one coefficient vector of
 // (c^L * max rank) entries per stage for each of up to 4 RHS per pass; larger needs
 // are rejected with MBF_ERR_INVALID.  Every call on a device
@@ -28,7 +28,7 @@
 namespace {
 
 constexpr size_t kStaticScratchBytes = size_t(4) << 20;
-constexpr size_t kBarrierBytes = 256;
+constexpr size_t kHeadBytes = 256;   // unused, before the counters: part of the size limit callers know
 constexpr int kMaxDevices = 64;
 
 // Device-side scratch.  In host code this name is only a host-side stand-in for
@@ -64,7 +64,7 @@ void apply_static_impl(mbf_op_s* op, const void* g, void* u, int64_t nrhs, void*
     mbf::fail(MBF_ERR_INVALID, "FP32 SIMT path unavailable: " + op->simt_unavailable);
   const int nrb = nrhs >= 4 ? 4 : (nrhs >= 2 ? 2 : 1);
   const size_t vec_bytes = size_t(op->positions) * size_t(nrb) * sizeof(float2);
-  const size_t sync_bytes = kBarrierBytes + mbf::counter_bytes(op->plan);
+  const size_t sync_bytes = kHeadBytes + mbf::counter_bytes(op->plan);
   const size_t need = sync_bytes + size_t(op->plan.n_stages) * vec_bytes;
   if (need > kStaticScratchBytes)
     mbf::fail(MBF_ERR_INVALID, "operator needs " + std::to_string(need) + " bytes of scratch for " +
@@ -93,7 +93,7 @@ void apply_static_impl(mbf_op_s* op, const void* g, void* u, int64_t nrhs, void*
   a.out = static_cast<float2*>(u);
   a.in_len = op->n_in;
   a.out_len = op->n_out;
-  a.counters = reinterpret_cast<unsigned*>(base + kBarrierBytes);   // cleared by each launch
+  a.counters = reinterpret_cast<unsigned*>(base + kHeadBytes);   // cleared by each launch
   a.bufs = reinterpret_cast<float2*>(base + sync_bytes);     // one vector per stage
   a.buf_stride = op->positions * nrb;
   a.status = op->ws.status;

@@ -37,7 +37,6 @@
 // stores, 2300 cycles, overlaps the other set's and covers all groups stored by then (it
 // paced the kernel at one group per fence).  122 -> 100 us; n = 128, r = 16, 20 RHS: 87 -> 61.
 #include <cuda_runtime.h>
-#include <cuda_bf16.h>
 
 #include <algorithm>
 #include <cstdint>
@@ -149,30 +148,9 @@ __device__ __forceinline__ uint4 tf32x4(const float* y) {
 __device__ __forceinline__ void mma_commit(uint64_t* b) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(b)) : "memory");
 }
-__device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-// Named barrier that also ORs a flag over the participating threads, so that every
-// thread takes the same branch after it.
-__device__ __forceinline__ bool named_sync_or(int id, int n, bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"(uint32_t(v)), "r"(id), "r"(n)
-      : "memory");
-  return r != 0;
-}
 
-
-// 16 consecutive TMEM columns of this thread's lane (one row of the accumulator),
-// written straight into the 16 FP32 registers (b32 operands take any 32-bit register).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
-        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
-      : "r"(taddr));
-}
-// 32 consecutive TMEM columns of this thread's lane.
+// 32 consecutive TMEM columns of this thread's lane (one row of the accumulator), written
+// straight into the FP32 registers (b32 operands take any 32-bit register).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -254,8 +232,6 @@ __device__ __forceinline__ int pat_group(int pat, int64_t P, const TCStage& s, i
   const int64_t q = P / s.ch;
   return int((P - q * s.ch) * s.B + q / c);
 }
-
-__device__ __forceinline__ uint16_t bf16_bits(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
 
 // Bounded wait on an mbarrier phase.  Returns false on timeout or abort.
 __device__ __forceinline__ bool wait_bar(uint64_t* b, uint32_t ph, volatile int* abort) {

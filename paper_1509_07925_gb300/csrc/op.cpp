@@ -1604,9 +1604,8 @@ mbf_status mbf_op_check(mbf_op_t op, void* stream) {
     cuda_check(cudaMemcpy(&st, op->ws.status, sizeof(int), cudaMemcpyDeviceToHost), "read status");
     if (st != ST_OK) {
       cuda_check(zero_now(op->ws.status, sizeof(int)), "clear status");
-      static const char* names[] = {"ok", "grid barrier", "full mbarrier", "empty mbarrier", "bad item",
-                                    "dependency counter"};
-      fail(MBF_ERR_TIMEOUT, std::string("device wait gave up: ") + (st >= 0 && st <= 5 ? names[st] : "unknown"));
+      static const char* names[] = {"ok", "full mbarrier", "empty mbarrier", "bad item", "dependency counter"};
+      fail(MBF_ERR_TIMEOUT, std::string("device wait gave up: ") + (st >= 0 && st <= 4 ? names[st] : "unknown"));
     }
   });
 }
