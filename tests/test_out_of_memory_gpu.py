@@ -35,13 +35,16 @@ def _refused(bd, op):
 
 
 def test_a_refused_allocation_leaves_no_error_behind(bd_op):
-    """Launches check the CUDA runtime's last error: it must not still be the refusal."""
+    """A later check of the CUDA runtime's last error, as launches are followed by, must not
+    find the refusal, which the call has reported."""
     bd, op = bd_op
+    cudart = C.CDLL(f"libcudart.so.{torch.version.cuda.split('.')[0]}")
     g = torch.from_numpy(complex_normal(N * N, 64, seed=81).astype(np.complex64)).cuda()
     out = [torch.zeros_like(g) for _ in range(2)]
     st = torch.cuda.current_stream().cuda_stream
     op.apply(g.data_ptr(), out[0].data_ptr(), 64, bd.MBF_PREC_BF16X3, st)
     _refused(bd, op)
+    assert cudart.cudaPeekAtLastError() == 0
     op.apply(g.data_ptr(), out[1].data_ptr(), 64, bd.MBF_PREC_BF16X3, st)
     op.check(st)
     assert torch.equal(torch.view_as_real(out[0]), torch.view_as_real(out[1]))
