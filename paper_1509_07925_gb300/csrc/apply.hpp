@@ -106,7 +106,8 @@ constexpr int kTcNR = 64;        // RHS of a tensor-core panel (MMAs of M = 128)
 // buffers take half the shared memory (so the tile ring is deeper) and its leaf products
 // are half as many.  n = 128, r = 16 with 20 RHS: 84 us with panels of 64, 77 with 32;
 // multiscale n = 128 with 32 RHS: 324 and 280; 3-D n = 32, r = 32 with 32 RHS: 252 (two ring
-// slots beside one panel buffer) and 173 (four).
+// slots beside one panel buffer) and 173 (four).  On a few dozen groups it may be the slower
+// one by a microsecond: n = 64, L = 4, r = 24 with 20 RHS 35.5 and 36.9, r = 64 76.7 and 60.1.
 constexpr int kTcNRHalf = 32;
 MBF_HD int64_t split_block_bytes(int R8, int nr = kTcNR) { return int64_t(R8) * nr * 8; }
 // With TF32 operands the same block holds FP32 (TF32-rounded) values instead, byte

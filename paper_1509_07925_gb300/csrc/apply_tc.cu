@@ -248,7 +248,7 @@ __device__ __forceinline__ bool wait_bar(uint64_t* b, uint32_t ph, volatile int*
 
 constexpr int kTcThreads = 480;   // 15 warps (roles above)
 constexpr int kAProducers = 2;    // lanes of warp 0 issuing the tile copies
-constexpr int kMaxXBufs = 3;      // panel buffers at most (the autotuner picks 2 or 3)
+constexpr int kMaxXBufs = 3;      // panel buffers at most (creation picks 1 or 2, the autotuner up to 3)
 constexpr int kTcChunk = 16;   // accumulator columns per epilogue step
 
 // TF32: the vectors between stages are TF32 blocks (apply.hpp) and the tiles two FP32

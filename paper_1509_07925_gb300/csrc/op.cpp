@@ -710,7 +710,10 @@ mbf_op_s* op_create(const mbf_factors_t& f) {
         if (smem(2) > size_t(optin)) fail(MBF_ERR_INVALID, "tiles too large for the tensor path");
         nsa = 2;   // a multiple of the tile stream's producer lanes (2)
         while (nsa + 2 <= 16 && smem(nsa + 2) <= size_t(optin)) nsa += 2;
-        if (nsa == 2 && nxb == 2) {   // wide tiles: a deeper ring is worth more than the second panel
+        // wide tiles: a deeper ring is worth more than the second panel (us with two buffers and
+        // two slots, with one and six or four: panels of 64, tiles of 160 rows, n = 64, L = 4 55.7,
+        // 45.5, polar n = 128, L = 6 331, 251; panels of 32, 256 rows, n = 64, L = 4 77.1, 60.2)
+        if (nsa == 2 && nxb == 2) {
           nxb = 1;
           while (nsa + 2 <= 16 && smem(nsa + 2) <= size_t(optin)) nsa += 2;
           if (nsa == 2) nxb = 2;
