@@ -205,8 +205,11 @@ mbf_status mbf_op_create(const mbf_factors_t* f, mbf_op_t* out);
 /* The device bytes the packed factors of f will take, without a device: *simt_bytes the
  * FP32 SIMT arena and its item table, *tensor_bytes the split-BF16 tiles (0 when the
  * tensor path cannot take the operator).  The tensor adjoint adds tensor_bytes again on
- * its first use, TF32 applies likewise; workspaces come on top.  Packs on the host to
- * count (host memory and time of the packing itself).  Either pointer may be NULL. */
+ * its first use, TF32 applies likewise; workspaces come on top (FP32: 8 vectors, or 4
+ * where the device has no room for 8, of c^L * max rank complex64 for each of the
+ * 2 (L - L/2) + 1 stages but the last; again for each further batch that a server has in
+ * flight).  Packs on the host to count (host memory and time of the packing itself).
+ * Either pointer may be NULL. */
 mbf_status mbf_factors_device_bytes(const mbf_factors_t* f, int64_t* simt_bytes, int64_t* tensor_bytes);
 /* mbf_build_factors + mbf_op_create + mbf_factors_destroy, then the error estimate
  * below on 256 sampled outputs (needs the device; kept for mbf_op_info). */

@@ -31,7 +31,7 @@
 // n = 64, L = 6 with 1 and 2 RHS, r = 4 44.5 / 46.5 -> 43.6 / 46.2 us, r = 8 46.7 / 50.6 ->
 // 43.7 / 48.7; n = 256, L = 8, r = 4 654 / 776 -> 655 / 757 (the many lines side by side of such
 // blocks are added in pairs; one after another they took r = 4 to 55.1 / 61.2 and 876 / 1002).
-// The kernels of 4 and 8 RHS spill 40 to 160 bytes (128 registers a thread).
+// The kernels of 4 and 8 RHS spill 40 to 120 bytes (128 registers a thread).
 #include <cuda_runtime.h>
 
 #include <algorithm>
